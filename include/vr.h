@@ -76,12 +76,12 @@ typedef enum { VR_COMPOSITE = 0, VR_MIP = 1 } vr_mode;
  *   its cells staged in shared memory, one pass per visibility key of the cells
  *   within the brick (tables of more than 256 entries: whole-brick marches from
  *   global memory, the same image up to rounding).  VR_MIP: as VR_PATH_BRICK.
- * VR_PATH_LAYERED: composite by bricks, one visibility layer per launch, each
- *   pixel's running (C, T) carried from layer to layer with per-sample early
- *   termination (the same image as VR_PATH_RAY); bricks of terminated pixels
- *   are skipped.  VR_MIP: as VR_PATH_BRICK.
- * Both read back per-view layer sizes (a host synchronisation), so graph mode
- * does not apply to them.
+ * VR_PATH_LAYERED: composite by bricks in visibility order, each pixel's running
+ *   (C, T) carried from brick to brick with per-sample early termination (the
+ *   same image as VR_PATH_RAY); bricks behind a terminated pixel are skipped.
+ *   VR_MIP: as VR_PATH_BRICK.
+ * The composite of VR_PATH_SORTLAST reads back the partial images' size (a host
+ * synchronisation); graph mode does not apply to either composite.
  * VR_PATH_AUTO (default): VR_PATH_BRICK for VR_MIP when available, else
  *   VR_PATH_RAY.  Every path computes the same discretisation. */
 typedef enum {

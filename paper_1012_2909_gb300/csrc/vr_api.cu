@@ -98,8 +98,6 @@ struct vr_ctx {
     long long partial_cap = 0;
     float4* state = nullptr;
     long long state_cap = 0;
-    int* host_rb = nullptr;        // page-locked read-back buffer
-    int host_rb_cap = 0;
     float* tf_partials = nullptr;  // adjoint: per-block table-gradient partials
     size_t tf_partials_n = 0;
     int* status_host = nullptr;    // mapped, page-locked device status word
@@ -405,7 +403,6 @@ vr_status vr_destroy(vr_ctx* ctx) {
                         (void*)ctx->partial_used, (void*)ctx->partial, (void*)ctx->state,
                         (void*)ctx->dist_ids, (void*)ctx->dist_foot})
             if (p) cudaFree(p);
-        if (ctx->host_rb) cudaFreeHost(ctx->host_rb);
         if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
         if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
         if (ctx->status_host) cudaFreeHost(ctx->status_host);
@@ -740,7 +737,10 @@ TFDev tf_dev(const vr_ctx* ctx) {
     return t;
 }
 
-vr_status render_ray(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max, cudaStream_t s) {
+// Image order: the marcher, or (layered, composite only) its form that walks the bricks
+// as parts with carried state.
+vr_status render_ray(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max, cudaStream_t s,
+                     bool layered = false) {
     const int ncams = (int)ctx->cams.size();
     const int nbatch = (ncams + kMaxLaunchCams - 1) / kMaxLaunchCams;
     VR_CK(cudaMemsetAsync(ctx->work, 0, sizeof(int) * nbatch, s), "vr_render: scheduler reset");
@@ -759,7 +759,10 @@ vr_status render_ray(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
     P.ert = (float)ctx->opt.ert;
     P.samples = ctx->sample_counter;
     const int block = ctx->tune.block;
-    const int grid = ctx->num_sms * march_blocks_per_sm(ctx->dtype, mode, P.vol.pool1 != nullptr, block) * block / 32;
+    const bool paired = P.vol.pool1 != nullptr;
+    const int per_sm = layered ? layered_blocks_per_sm(ctx->dtype, paired, block)
+                               : march_blocks_per_sm(ctx->dtype, mode, paired, block);
+    const int grid = ctx->num_sms * per_sm * block / 32;
     const long long img = (long long)P.width * P.height;
     if (ctx->ev_start) VR_CK(cudaEventRecord(ctx->ev_start, s), "vr_render: profiling event");
     for (int b = 0; b < nbatch; ++b) {
@@ -771,7 +774,9 @@ vr_status render_ray(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
         P.work = ctx->work + b;
         const int tiles = P.tiles_x * P.tiles_y * P.ncams;  // one warp per tile
         const int blocks = std::max(1, std::min(grid / (block / 32), (tiles + block / 32 - 1) / (block / 32)));
-        VR_CK(launch_march(P, ctx->dtype, blocks, block, s), "vr_render: march launch");
+        VR_CK(layered ? launch_march_layered(P, ctx->dtype, blocks, block, s)
+                      : launch_march(P, ctx->dtype, blocks, block, s),
+              "vr_render: march launch");
     }
     if (ctx->ev_stop) VR_CK(cudaEventRecord(ctx->ev_stop, s), "vr_render: profiling event");
     return VR_OK;
@@ -931,11 +936,9 @@ vr_status staged_partials(vr_ctx* ctx, const CamDev& cd, const SortParams& sp, i
     return VR_OK;
 }
 
-// Composite in object order.  carried = false: per-brick partial images from
-// T = 1 folded in visibility order (no early termination).  carried = true:
-// one visibility layer of bricks per launch, each pixel's running (C, T)
-// carried through with per-sample early termination.
-vr_status render_bricks_composite(vr_ctx* ctx, float* out_rgba, cudaStream_t s, bool carried) {
+// Sort-last composite: per-brick partial images from T = 1 folded in visibility
+// order (no early termination).
+vr_status render_sortlast_composite(vr_ctx* ctx, float* out_rgba, cudaStream_t s) {
     const int W = ctx->cams[0].width, H = ctx->cams[0].height;
     const long long img = (long long)W * H;
     const long long nbricks = (long long)ctx->nbx * ctx->nby * ctx->nbz;
@@ -956,22 +959,17 @@ vr_status render_bricks_composite(vr_ctx* ctx, float* out_rgba, cudaStream_t s, 
         ctx->sort_bricks = nbricks + 1;
     }
     if (!ctx->partial_used) VR_CK(cudaMalloc(&ctx->partial_used, sizeof(unsigned long long)), "sort-last scratch");
-    if (carried) {
-        st = grow(ctx, ctx->state, ctx->state_cap, img, "layered state");
-        if (st != VR_OK) return st;
-    }
     SortParams sp;
     std::memset(&sp, 0, sizeof(sp));
     sp.vol = vol_dev(ctx);
     sp.tf = tf_dev(ctx);
     split(ctx->opt.step, sp.step, sp.step_lo);
-    sp.ert = carried ? (float)ctx->opt.ert : 2.0f;
+    sp.ert = 2.0f;
     sp.krange = ctx->krange;
     sp.foot = ctx->foot;
     sp.order = ctx->order;
     sp.tile_start = ctx->tile_start;
     sp.partial_used = ctx->partial_used;
-    sp.state = ctx->state;
     PixelParams pp;
     std::memset(&pp, 0, sizeof(pp));
     pp.vol = sp.vol;
@@ -996,13 +994,6 @@ vr_status render_bricks_composite(vr_ctx* ctx, float* out_rgba, cudaStream_t s, 
             VR_CK(cudaMalloc(&ctx->layer_buf, sizeof(int) * 3 * (size_t)(L + 1)), "sort-last scratch");
             ctx->layer_cap = L + 1;
         }
-        if (L + 2 > ctx->host_rb_cap) {
-            if (ctx->host_rb) cudaFreeHost(ctx->host_rb);
-            ctx->host_rb = nullptr;
-            ctx->host_rb_cap = 0;
-            VR_CK(cudaHostAlloc(&ctx->host_rb, sizeof(int) * (size_t)(L + 4), cudaHostAllocDefault), "read-back");
-            ctx->host_rb_cap = L + 4;
-        }
         sp.max_layers = L;
         sp.layer_count = ctx->layer_buf;
         sp.layer_start = ctx->layer_buf + (L + 1);
@@ -1013,45 +1004,27 @@ vr_status render_bricks_composite(vr_ctx* ctx, float* out_rgba, cudaStream_t s, 
         VR_CK(cudaMemsetAsync(sp.layer_count, 0, sizeof(int) * (size_t)L, s), "vr_render: reset");
         VR_CK(cudaMemsetAsync(sp.partial_used, 0, sizeof(unsigned long long), s), "vr_render: reset");
         VR_CK(launch_brick_footprints(sp, s), "vr_render: brick footprints");
-        // read back the layer starts and the partial-image size (host decides the launches)
-        VR_CK(cudaMemcpyAsync(ctx->host_rb, sp.layer_start, sizeof(int) * (size_t)(L + 1), cudaMemcpyDeviceToHost, s),
-              "vr_render: read-back");
+        // read back the partial images' size (the host allocates them)
         unsigned long long used = 0;
         VR_CK(cudaMemcpyAsync(&used, sp.partial_used, sizeof(used), cudaMemcpyDeviceToHost, s), "vr_render: read-back");
         VR_CK(cudaStreamSynchronize(s), "vr_render: read-back");
-        if (!carried) {
-            vr_status g = grow(ctx, ctx->partial, ctx->partial_cap, (long long)std::max<unsigned long long>(used, 1),
-                               "partial images");
-            if (g != VR_OK) return g;
-            sp.partial = ctx->partial;
-            sp.work = ctx->work;
-            if (ctx->ev_start && ci == 0) VR_CK(cudaEventRecord(ctx->ev_start, s), "vr_render: profiling event");
-            bool staged = false;
-            st = staged_partials(ctx, cd, sp, VR_COMPOSITE, nullptr, 0, (long long)used, s, &staged);
-            if (st != VR_OK) return st;
-            if (!staged) {
-                VR_CK(launch_tile_scan(sp, s), "vr_render: tile prefix");
-                VR_CK(cudaMemsetAsync(sp.work, 0, sizeof(int), s), "vr_render: scheduler reset");
-                VR_CK(launch_brick_partial(sp, ctx->dtype, false, 0, L, grid, s), "vr_render: partial images");
-            }
-            if (ctx->ev_stop && ci + 1 == ctx->cams.size())
-                VR_CK(cudaEventRecord(ctx->ev_stop, s), "vr_render: profiling event");
-            VR_CK(launch_sortlast_fold(sp, s), "vr_render: sort-last fold");
-        } else {
+        vr_status g = grow(ctx, ctx->partial, ctx->partial_cap, (long long)std::max<unsigned long long>(used, 1),
+                           "partial images");
+        if (g != VR_OK) return g;
+        sp.partial = ctx->partial;
+        sp.work = ctx->work;
+        if (ctx->ev_start && ci == 0) VR_CK(cudaEventRecord(ctx->ev_start, s), "vr_render: profiling event");
+        bool staged = false;
+        st = staged_partials(ctx, cd, sp, VR_COMPOSITE, nullptr, 0, (long long)used, s, &staged);
+        if (st != VR_OK) return st;
+        if (!staged) {
             VR_CK(launch_tile_scan(sp, s), "vr_render: tile prefix");
-            VR_CK(launch_state_init(sp, s), "vr_render: state init");
-            int slot = 0;
-            if (ctx->ev_start && ci == 0) VR_CK(cudaEventRecord(ctx->ev_start, s), "vr_render: profiling event");
-            for (int l = 0; l < L; ++l) {
-                if (ctx->host_rb[l + 1] == ctx->host_rb[l]) continue;  // empty layer
-                sp.work = ctx->work + (slot++ % ctx->work_slots);
-                VR_CK(cudaMemsetAsync(sp.work, 0, sizeof(int), s), "vr_render: scheduler reset");
-                VR_CK(launch_brick_partial(sp, ctx->dtype, true, l, l + 1, grid, s), "vr_render: layer");
-            }
-            if (ctx->ev_stop && ci + 1 == ctx->cams.size())
-                VR_CK(cudaEventRecord(ctx->ev_stop, s), "vr_render: profiling event");
-            VR_CK(launch_state_finish(sp, s), "vr_render: state finish");
+            VR_CK(cudaMemsetAsync(sp.work, 0, sizeof(int), s), "vr_render: scheduler reset");
+            VR_CK(launch_brick_partial(sp, ctx->dtype, false, 0, L, grid, s), "vr_render: partial images");
         }
+        if (ctx->ev_stop && ci + 1 == ctx->cams.size())
+            VR_CK(cudaEventRecord(ctx->ev_stop, s), "vr_render: profiling event");
+        VR_CK(launch_sortlast_fold(sp, s), "vr_render: sort-last fold");
     }
     return VR_OK;
 }
@@ -1453,8 +1426,8 @@ vr_path resolve_path(const vr_ctx* ctx, vr_mode mode) {
 vr_status render_dispatch(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max, cudaStream_t s) {
     if (ctx->ooc) return render_ooc(ctx, mode, out_rgba, out_max, s);
     vr_path path = resolve_path(ctx, mode);
-    if ((path == VR_PATH_SORTLAST || path == VR_PATH_LAYERED) && mode == VR_COMPOSITE)
-        return render_bricks_composite(ctx, out_rgba, s, path == VR_PATH_LAYERED);
+    if (path == VR_PATH_SORTLAST && mode == VR_COMPOSITE) return render_sortlast_composite(ctx, out_rgba, s);
+    if (path == VR_PATH_LAYERED && mode == VR_COMPOSITE) return render_ray(ctx, mode, out_rgba, nullptr, s, true);
     if (path == VR_PATH_SORTLAST || path == VR_PATH_LAYERED) path = VR_PATH_BRICK;  // MIP: order-free
     if (path == VR_PATH_BRICK) {
         if (mode != VR_MIP)

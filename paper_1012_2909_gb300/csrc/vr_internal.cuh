@@ -188,6 +188,10 @@ cudaError_t launch_repack(const float* src, long long src_z0, long long src_plan
 // The marcher reads x-neighbour pairs with one load when p.vol.pool1 is set.
 cudaError_t launch_march(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s);
 int march_blocks_per_sm(vr_dtype dt, int mode, bool paired, int block);
+// Layered composite of a cube in core: as launch_march, the samples owned and
+// positioned brick by brick as in launch_brick_partial.
+cudaError_t launch_march_layered(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s);
+int layered_blocks_per_sm(vr_dtype dt, bool paired, int block);
 cudaError_t launch_pixel_setup(const PixelParams& p, cudaStream_t s);
 cudaError_t launch_mip_finalize(const PixelParams& p, cudaStream_t s);
 // `cells` is per-context scratch of brick_cells_bytes(units) bytes (a counter and the

@@ -18,10 +18,13 @@
 //   * with P.mode == VR_MIP the partial image of a brick is the maximum of its
 //     samples per pixel (-inf without samples) and the fold takes the maximum,
 //     then the transfer function;
-//   * k_brick_partial<CARRIED>: the same march continuing each pixel's running
-//     (C, T) with per-sample early termination, one visibility layer of bricks
-//     per launch (no two bricks of a layer own samples of the same ray), and
-//     bricks of terminated pixels skipped.
+//   * k_march_layered (cube in core): one thread per ray over its bricks in
+//     visibility order, its running (C, T) in registers, with per-sample early
+//     termination;
+//   * k_brick_partial<CARRIED> (streamed cubes): the same march continuing each
+//     pixel's running (C, T), one visibility layer of bricks per launch (no two
+//     bricks of a layer own samples of the same ray), and bricks of terminated
+//     pixels skipped.
 //
 // Visibility: the brick index along a ray moves monotonically away from the
 // eye's brick index e on every axis, so the key sum_a |b_a - e_a|
@@ -30,6 +33,7 @@
 // partition as the cell pass, clipped to the ray's sample range from the
 // pixel set-up.
 #include <algorithm>
+#include <climits>
 
 #include "vr_device.cuh"
 #include "vr_ff.cuh"
@@ -143,6 +147,64 @@ __global__ void k_layer_scatter(const __grid_constant__ SortParams P) {
     }
 }
 
+// FP32 origin o and step vector e of the ray of pixel centre (sx, sy): the numbers
+// that decide which brick owns a sample.
+__device__ __forceinline__ void ray_fp32(const CamFF& c, float sx, float sy, float step, float o[3], float e[3]) {
+    float V[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) V[a] = fmaf(sy, c.by_hi[a], fmaf(sx, c.bx_hi[a], c.base_hi[a]));
+    if (c.type == 1) {
+        const float inv = rsqrtf(V[0] * V[0] + V[1] * V[1] + V[2] * V[2]) * step;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            o[a] = c.org_hi[a];
+            e[a] = V[a] * inv;
+        }
+    } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            o[a] = V[a];
+            e[a] = c.dir_hi[a] * step;
+        }
+    }
+}
+
+// The same ray in float-float, for the sample positions O + k E.
+__device__ __forceinline__ void ray_ff(const CamFF& c, float sx, float sy, ff step, ff O[3], ff E[3]) {
+    if (c.type == 1) {
+        ff V[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            V[a] = ff_add(ff_add(ff{c.base_hi[a], c.base_lo[a]}, ff_mul_f(ff{c.bx_hi[a], c.bx_lo[a]}, sx)),
+                          ff_mul_f(ff{c.by_hi[a], c.by_lo[a]}, sy));
+            O[a] = ff{c.org_hi[a], c.org_lo[a]};
+        }
+        const ff n2 = ff_add(ff_add(ff_mul(V[0], V[0]), ff_mul(V[1], V[1])), ff_mul(V[2], V[2]));
+        const ff r = ff_rsqrt(n2);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) E[a] = ff_mul(ff_mul(V[a], r), step);
+    } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            O[a] = ff_add(ff_add(ff{c.base_hi[a], c.base_lo[a]}, ff_mul_f(ff{c.bx_hi[a], c.bx_lo[a]}, sx)),
+                          ff_mul_f(ff{c.by_hi[a], c.by_lo[a]}, sy));
+            E[a] = ff_mul(ff{c.dir_hi[a], c.dir_lo[a]}, step);
+        }
+    }
+}
+
+// Slot coordinate of sample k along one axis of the brick with index b.
+__device__ __forceinline__ float slot_coord(ff O, ff E, ff fk, int b, int B) {
+    const ff p = ff_add(O, ff_mul(E, fk));
+    return __fadd_rn(__fsub_rn(p.hi, (float)(b * B)), p.lo) + 0.5f;
+}
+
+// Sample index at which a ray crosses the plane X (any fixed reciprocal keeps it
+// deterministic and monotone in X).
+__device__ __forceinline__ float plane_kappa(float X, float o, float inv) {
+    return __fmul_rn(__fsub_rn(X, o), inv);
+}
+
 // Samples of pixel (px, py) owned by brick (bx,by,bz): [ka, kb) and the
 // float-float anchored slot coordinate of sample ka; false if none.
 __device__ __forceinline__ bool brick_segment(const SortParams& P, int px, int py, int2 kr, int bx, int by,
@@ -150,25 +212,7 @@ __device__ __forceinline__ bool brick_segment(const SortParams& P, int px, int p
     const CamFF& c = P.cam;
     const float sx = (float)px + 0.5f, sy = (float)py + 0.5f;
     float o[3], e[3];
-    {
-        float V[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) V[a] = fmaf(sy, c.by_hi[a], fmaf(sx, c.bx_hi[a], c.base_hi[a]));
-        if (c.type == 1) {
-            const float inv = rsqrtf(V[0] * V[0] + V[1] * V[1] + V[2] * V[2]) * P.step;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                o[a] = c.org_hi[a];
-                e[a] = V[a] * inv;
-            }
-        } else {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                o[a] = V[a];
-                e[a] = c.dir_hi[a] * P.step;
-            }
-        }
-    }
+    ray_fp32(c, sx, sy, P.step, o, e);
     const int B = P.vol.B;
     const int bi[3] = {bx, by, bz};
     const int nb[3] = {P.vol.nbx, P.vol.nby, P.vol.nbz};
@@ -180,8 +224,8 @@ __device__ __forceinline__ bool brick_segment(const SortParams& P, int px, int p
         const float xl = (float)(bi[a] * B), xh = (float)((bi[a] + 1) * B);
         if (e[a] != 0.f) {
             const float inv = __fdividef(1.0f, e[a]);
-            const float kl = __fmul_rn(__fsub_rn(xl, o[a]), inv);
-            const float kh = __fmul_rn(__fsub_rn(xh, o[a]), inv);
+            const float kl = plane_kappa(xl, o[a], inv);
+            const float kh = plane_kappa(xh, o[a], inv);
             float a0, a1;
             if (e[a] > 0.f) {
                 a0 = first ? -1e9f : kl;
@@ -202,31 +246,11 @@ __device__ __forceinline__ bool brick_segment(const SortParams& P, int px, int p
     kb = min((int)ceilf(khi), kr.y);
     if (ka >= kb) return false;
     ff E[3], O[3];
-    if (c.type == 1) {
-        ff V[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            V[a] = ff_add(ff_add(ff{c.base_hi[a], c.base_lo[a]}, ff_mul_f(ff{c.bx_hi[a], c.bx_lo[a]}, sx)),
-                          ff_mul_f(ff{c.by_hi[a], c.by_lo[a]}, sy));
-            O[a] = ff{c.org_hi[a], c.org_lo[a]};
-        }
-        const ff n2 = ff_add(ff_add(ff_mul(V[0], V[0]), ff_mul(V[1], V[1])), ff_mul(V[2], V[2]));
-        const ff r = ff_rsqrt(n2);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) E[a] = ff_mul(ff_mul(V[a], r), ff{P.step, P.step_lo});
-    } else {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            O[a] = ff_add(ff_add(ff{c.base_hi[a], c.base_lo[a]}, ff_mul_f(ff{c.bx_hi[a], c.bx_lo[a]}, sx)),
-                          ff_mul_f(ff{c.by_hi[a], c.by_lo[a]}, sy));
-            E[a] = ff_mul(ff{c.dir_hi[a], c.dir_lo[a]}, ff{P.step, P.step_lo});
-        }
-    }
+    ray_ff(c, sx, sy, ff{P.step, P.step_lo}, O, E);
     const ff fk = ff_of_int(ka);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const ff p = ff_add(O[a], ff_mul(E[a], fk));
-        g[a] = __fadd_rn(__fsub_rn(p.hi, (float)(bi[a] * B)), p.lo) + 0.5f;  // slot coordinate
+        g[a] = slot_coord(O[a], E[a], fk, bi[a], B);
         e32[a] = E[a].hi;
     }
     return true;
@@ -248,13 +272,10 @@ __global__ void k_tile_scan(const __grid_constant__ SortParams P) {
 
 // One warp per (brick, 8 x 4 tile of its rectangle); one thread per pixel.
 // Bricks of the ordered positions [start of layer l0, start of layer l1).
-// PAIRED (16-bit stores with the shifted copy, layered path): each x-neighbour
-// pair of a trilinear fetch is one 32-bit load (fetch_trilinear_pair, the same
-// values bit for bit), halving the gathers (survey layered composite 3.03 ->
-// 2.71 ms).  The independent partials march whole bricks without termination,
-// like MIP rays, and reading both copies there measured no faster (9.6-10.1 ->
-// 10.2 ms): they read the store alone.
-template <typename T, bool CARRIED, bool PAIRED>
+// The store alone is read: streamed cubes (CARRIED) keep no shifted copy, and the
+// independent partials march whole bricks without termination, like MIP rays,
+// where reading both copies measured no faster (9.6-10.1 -> 10.2 ms).
+template <typename T, bool CARRIED>
 __global__ void __launch_bounds__(128)
 k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer_end) {
     __shared__ float4 s_tf[kMaxTF];
@@ -268,12 +289,7 @@ k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer
     const int end = P.sub_order ? P.sub_n : P.layer_start[layer_end];
     const int t0 = tile_start[first], t1 = tile_start[end];
     const T* __restrict__ pool = static_cast<const T*>(P.vol.pool);
-    const T* __restrict__ pool1 = static_cast<const T*>(P.vol.pool1);
     const float ert = P.ert;
-    auto fetch = [&](const T* slot, const T* slot1, float gx, float gy, float gz) {
-        if constexpr (PAIRED) return fetch_trilinear_pair<T>(slot, slot1, P.vol, gx, gy, gz);
-        else return fetch_trilinear<T>(slot, P.vol, gx, gy, gz);
-    };
     for (;;) {
         int item = 0;
         if (lane == 0) item = atomicAdd(P.work, 1);
@@ -314,10 +330,10 @@ k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer
             if (any) {
                 const long long base = (long long)P.vol.table[b] * P.vol.slot_elems;
                 const T* slot = pool + base;
-                const T* slot1 = PAIRED ? pool1 + base : nullptr;
                 for (int j = 0; j < kb - ka; ++j) {
                     const float fj = (float)j;
-                    m = fmaxf(m, fetch(slot, slot1, fmaf(fj, e[0], g[0]), fmaf(fj, e[1], g[1]), fmaf(fj, e[2], g[2])));
+                    m = fmaxf(m, fetch_trilinear<T>(slot, P.vol, fmaf(fj, e[0], g[0]), fmaf(fj, e[1], g[1]),
+                                                    fmaf(fj, e[2], g[2])));
                 }
             }
             const int rw = rect.z - rect.x + 1;
@@ -327,12 +343,12 @@ k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer
         if (any) {
             const long long base = (long long)P.vol.table[b] * P.vol.slot_elems;
             const T* slot = pool + base;
-            const T* slot1 = PAIRED ? pool1 + base : nullptr;
             // at most ~4 B samples per brick: FP32 stepping from the float-float anchor
             // stays within 2e-5 voxel
             for (int j = 0; j < kb - ka; ++j) {
                 const float fj = (float)j;
-                const float v = fetch(slot, slot1, fmaf(fj, e[0], g[0]), fmaf(fj, e[1], g[1]), fmaf(fj, e[2], g[2]));
+                const float v = fetch_trilinear<T>(slot, P.vol, fmaf(fj, e[0], g[0]), fmaf(fj, e[1], g[1]),
+                                                   fmaf(fj, e[2], g[2]));
                 const float4 c = tf_lookup(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v);
                 const float w = Tr * c.w;
                 C0 = fmaf(w, c.x, C0);
@@ -348,6 +364,137 @@ k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer
             const int rw = rect.z - rect.x + 1;
             P.partial[f.offset + (long long)(py - rect.y) * rw + (px - rect.x)] = make_float4(C0, C1, C2, Tr);
         }
+    }
+}
+
+// Composite by bricks with carried state, for a cube in core: one thread per ray
+// walks the ray's bricks in visibility order with its (C, T) in registers, with
+// per-sample early termination.  Ownership and positions are those of
+// brick_segment, so the image equals, bit for bit, the one of one launch of
+// k_brick_partial<CARRIED> per visibility layer.
+//
+// Bound by L1 data wavefronts, like the image-order marcher: a ray stops in a front
+// shell that stays in the caches.  One launch per layer left 14-22 % of the warps
+// active (27 launches on the survey cube), set a ray up again in every brick,
+// carried its state through memory, and needed the bricks' order on the host;
+// here a pixel's set-up is done once and U samples' fetches are in flight at a time.
+// Survey frame (1024 x 1024 x 2048, 1920 x 1080, BF16): 3.27 -> 0.51 ms.  With paired
+// loads U = 4, 5, 6, 8 took 0.538, 0.515, 0.507, 0.538 ms.
+constexpr int kLayeredUnroll = 4;
+constexpr int kLayeredUnrollPaired = 6;
+
+template <typename T, bool PAIRED>
+__global__ void __launch_bounds__(256, 2)
+k_march_layered(const __grid_constant__ MarchParams P) {
+    constexpr int U = PAIRED ? kLayeredUnrollPaired : kLayeredUnroll;
+    __shared__ float4 s_tf[kMaxTF];
+    for (int i = threadIdx.x; i < P.tf.n; i += blockDim.x) s_tf[i] = P.tf.tab[i];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int tiles_per_cam = P.tiles_x * P.tiles_y;
+    const int total = tiles_per_cam * P.ncams;
+    const T* __restrict__ pool = static_cast<const T*>(P.vol.pool);
+    const T* __restrict__ pool1 = static_cast<const T*>(P.vol.pool1);
+    const float ert = P.ert;
+    const int B = P.vol.B;
+    const int nb[3] = {P.vol.nbx, P.vol.nby, P.vol.nbz};
+    for (;;) {
+        int item = 0;
+        if (lane == 0) item = atomicAdd(P.work, 1);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if (item >= total) break;
+        const int cam = item / tiles_per_cam;
+        const int tile = item - cam * tiles_per_cam;
+        const int ty = tile / P.tiles_x, tx = tile - ty * P.tiles_x;
+        const int px = tx * P.tile_w + (lane % P.tile_w);
+        const int py = ty * P.tile_h + (lane / P.tile_w);
+        if (px >= P.width || py >= P.height) continue;  // ragged edge tile; the lane
+                                                        // rejoins at the next shuffle
+        const CamFF& c = P.cams[cam];
+        float C0 = 0.f, C1 = 0.f, C2 = 0.f, Tr = 1.f;
+        Ray r;
+        if (make_ray(c, px, py, P.vol, ff{P.step_hi, P.step_lo}, r)) {
+            const float sx = (float)px + 0.5f, sy = (float)py + 0.5f;
+            float o[3], e[3], inv[3];
+            ray_fp32(c, sx, sy, P.step_hi, o, e);
+            ff O[3], E[3];
+            ray_ff(c, sx, sy, ff{P.step_hi, P.step_lo}, O, E);
+            // b: the brick index that owns sample k; leave: the first sample past it
+            int b[3], leave[3];
+            auto crossing = [&](int a, int plane) {  // first sample at or past the plane
+                const float kap = plane_kappa((float)(plane * B), o[a], inv[a]);
+                return (int)ceilf(fminf(fmaxf(kap, -1e9f), 1e9f));
+            };
+            auto leaving = [&](int a) {
+                if (e[a] > 0.f) return b[a] == nb[a] - 1 ? INT_MAX : crossing(a, b[a] + 1);
+                if (e[a] < 0.f) return b[a] == 0 ? INT_MAX : crossing(a, b[a]);
+                return INT_MAX;
+            };
+            int k = r.k0;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                inv[a] = e[a] != 0.f ? __fdividef(1.0f, e[a]) : 0.f;
+                // near the owner, then moved to it by the same crossings that decide ownership
+                const float x = e[a] != 0.f ? fmaf((float)k, e[a], o[a]) : o[a];
+                b[a] = min(max((int)floorf(x) >> P.vol.log2B, 0), nb[a] - 1);
+                if (e[a] > 0.f) {
+                    while (b[a] > 0 && k < crossing(a, b[a])) --b[a];
+                } else if (e[a] < 0.f) {
+                    while (b[a] < nb[a] - 1 && k < crossing(a, b[a] + 1)) ++b[a];
+                }
+                leave[a] = leaving(a);
+                while (k >= leave[a]) {
+                    b[a] += e[a] > 0.f ? 1 : -1;
+                    leave[a] = leaving(a);
+                }
+            }
+            bool done = false;
+            while (k < r.k1 && !done) {
+                const int kb = min(r.k1, min(leave[0], min(leave[1], leave[2])));
+                const int brick = (b[2] * nb[1] + b[1]) * nb[0] + b[0];
+                if (!brick_transparent(P.vol, P.tf, brick)) {  // else opacity 0 throughout
+                    const long long base = (long long)P.vol.table[brick] * P.vol.slot_elems;
+                    const T* slot = pool + base;
+                    const T* slot1 = PAIRED ? pool1 + base : nullptr;
+                    const ff fk = ff_of_int(k);
+                    const float gx = slot_coord(O[0], E[0], fk, b[0], B), gy = slot_coord(O[1], E[1], fk, b[1], B),
+                                gz = slot_coord(O[2], E[2], fk, b[2], B);
+                    const int n = kb - k;
+                    for (int i = 0; i < n && !done; i += U) {
+                        float v[U];
+#pragma unroll
+                        for (int q = 0; q < U; ++q) {
+                            const float fj = (float)min(i + q, n - 1);
+                            const float x = fmaf(fj, E[0].hi, gx), y = fmaf(fj, E[1].hi, gy), z = fmaf(fj, E[2].hi, gz);
+                            if constexpr (PAIRED) v[q] = fetch_trilinear_pair<T>(slot, slot1, P.vol, x, y, z);
+                            else v[q] = fetch_trilinear<T>(slot, P.vol, x, y, z);
+                        }
+#pragma unroll
+                        for (int q = 0; q < U; ++q) {
+                            if (i + q >= n) break;
+                            const float4 t = tf_lookup(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v[q]);
+                            const float w = Tr * t.w;
+                            C0 = fmaf(w, t.x, C0);
+                            C1 = fmaf(w, t.y, C1);
+                            C2 = fmaf(w, t.z, C2);
+                            Tr = Tr * (1.f - t.w);
+                            if (1.f - Tr >= ert) {
+                                done = true;
+                                break;
+                            }
+                        }
+                    }
+                }
+                k = kb;
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    while (k >= leave[a]) {
+                        b[a] += e[a] > 0.f ? 1 : -1;
+                        leave[a] = leaving(a);
+                    }
+            }
+        }
+        P.out_rgba[((long long)cam * P.height + py) * P.width + px] = make_float4(C0, C1, C2, 1.f - Tr);
     }
 }
 
@@ -438,13 +585,7 @@ __global__ void k_state_finish(const __grid_constant__ SortParams P) {
 
 template <typename T, bool CARRIED>
 cudaError_t partial_t(const SortParams& p, int l0, int l1, int grid, cudaStream_t s) {
-    if constexpr (sizeof(T) == 2 && CARRIED) {
-        if (p.vol.pool1) {
-            k_brick_partial<T, CARRIED, true><<<grid, 128, 0, s>>>(p, l0, l1);
-            return cudaGetLastError();
-        }
-    }
-    k_brick_partial<T, CARRIED, false><<<grid, 128, 0, s>>>(p, l0, l1);
+    k_brick_partial<T, CARRIED><<<grid, 128, 0, s>>>(p, l0, l1);
     return cudaGetLastError();
 }
 
@@ -473,6 +614,28 @@ cudaError_t launch_brick_partial(const SortParams& p, vr_dtype dt, bool carried,
     if (dt == VR_F16) return carried ? partial_t<__half, true>(p, l0, l1, grid, s) : partial_t<__half, false>(p, l0, l1, grid, s);
     return carried ? partial_t<__nv_bfloat16, true>(p, l0, l1, grid, s)
                    : partial_t<__nv_bfloat16, false>(p, l0, l1, grid, s);
+}
+
+namespace {
+void* layered_ptr(vr_dtype dt, bool paired) {
+    if (dt == VR_F32) return reinterpret_cast<void*>(&k_march_layered<float, false>);
+    if (dt == VR_F16)
+        return paired ? reinterpret_cast<void*>(&k_march_layered<__half, true>)
+                      : reinterpret_cast<void*>(&k_march_layered<__half, false>);
+    return paired ? reinterpret_cast<void*>(&k_march_layered<__nv_bfloat16, true>)
+                  : reinterpret_cast<void*>(&k_march_layered<__nv_bfloat16, false>);
+}
+}  // namespace
+
+int layered_blocks_per_sm(vr_dtype dt, bool paired, int block) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, layered_ptr(dt, paired), block, 0) != cudaSuccess) return 1;
+    return n > 0 ? n : 1;
+}
+
+cudaError_t launch_march_layered(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s) {
+    void* args[] = {const_cast<MarchParams*>(&p)};
+    return cudaLaunchKernel(layered_ptr(dt, p.vol.pool1 != nullptr), dim3(grid), dim3(block), args, 0, s);
 }
 
 cudaError_t launch_sortlast_fold(const SortParams& p, cudaStream_t s) {
