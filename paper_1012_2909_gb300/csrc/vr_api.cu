@@ -456,22 +456,34 @@ vr_status vr_load_cube(vr_ctx* ctx, const float* src, int src_on_device, int64_t
     }
     VR_CK(cudaMemsetAsync(ctx->minmax, 0xff, sizeof(unsigned int) * nbricks, s), "vr_load_cube: memset");
     VR_CK(cudaMemsetAsync(ctx->minmax + nbricks, 0, sizeof(unsigned int) * nbricks, s), "vr_load_cube: memset");
+    const size_t plane = (size_t)nx * (size_t)ny;
+    const size_t stage_bytes = src_on_device ? 0 : plane * (size_t)std::min<long long>(ctx->rows, nz) * sizeof(float);
+    float* stage = nullptr;
+    if (!src_on_device)
+        VR_CK(cudaMallocAsync(reinterpret_cast<void**>(&stage), stage_bytes, s), "vr_load_cube: staging allocation");
+    if (storage != VR_F32 && !(ctx->opt.flags & VR_OPT_SINGLE_STORE)) {
+        // the copy shifted by one element (16-bit stores: an x-pair is one 32-bit load;
+        // FP32 pairs as 64-bit loads measured no faster), kept only when it fits in half
+        // of what is free beside the staging slab
+        size_t fr = 0, tot = 0;
+        if (cudaMemGetInfo(&fr, &tot) == cudaSuccess && pool_bytes <= (fr + stage_bytes) / 2 &&
+            cudaMalloc(&ctx->pool1, pool_bytes) != cudaSuccess) {
+            cudaGetLastError();  // not kept: the single-store path serves every render
+            ctx->pool1 = nullptr;
+        }
+    }
     VolDev v = vol_dev(ctx);
     if (src_on_device) {
-        for (int bz = 0; bz < ctx->nbz; ++bz)
-            VR_CK(launch_repack(src, 0, nz, bz, v, storage, ctx->pool, ctx->minmax, s), "vr_load_cube: repack");
+        VR_CK(launch_repack(src, 0, 0, ctx->nbz, v, storage, ctx->pool, ctx->pool1, ctx->minmax, s),
+              "vr_load_cube: repack");
     } else {
-        const size_t plane = (size_t)nx * (size_t)ny;
-        const long long maxp = std::min<long long>(ctx->rows, nz);
-        float* stage = nullptr;
-        VR_CK(cudaMallocAsync(reinterpret_cast<void**>(&stage), plane * maxp * sizeof(float), s),
-              "vr_load_cube: staging allocation");
         for (int bz = 0; bz < ctx->nbz; ++bz) {
             const long long z0 = std::max<long long>((long long)bz * B - 1, 0);
             const long long z1 = std::min<long long>((long long)bz * B + B + 1, nz);
             cudaError_t e = cudaMemcpyAsync(stage, src + (size_t)z0 * plane, plane * (z1 - z0) * sizeof(float),
                                             cudaMemcpyHostToDevice, s);
-            if (e == cudaSuccess) e = launch_repack(stage, z0, z1 - z0, bz, v, storage, ctx->pool, ctx->minmax, s);
+            if (e == cudaSuccess)
+                e = launch_repack(stage, z0, bz, 1, v, storage, ctx->pool, ctx->pool1, ctx->minmax, s);
             if (e != cudaSuccess) {
                 cudaFreeAsync(stage, s);
                 cudaStreamSynchronize(s);
@@ -482,25 +494,6 @@ vr_status vr_load_cube(vr_ctx* ctx, const float* src, int src_on_device, int64_t
         VR_CK(cudaFreeAsync(stage, s), "vr_load_cube: staging free");
     }
     VR_CK(cudaStreamSynchronize(s), "vr_load_cube: repack");
-    if (storage != VR_F32 && !(ctx->opt.flags & VR_OPT_SINGLE_STORE)) {
-        // the copy shifted by one element (16-bit stores: an x-pair is one 32-bit load;
-        // FP32 pairs as 64-bit loads measured no faster), kept only when it fits in half
-        // of what is free
-        size_t fr = 0, tot = 0;
-        if (cudaMemGetInfo(&fr, &tot) == cudaSuccess && pool_bytes <= fr / 2) {
-            if (cudaMalloc(&ctx->pool1, pool_bytes) == cudaSuccess) {
-                const size_t e = (size_t)ctx->elem;
-                VR_CK(cudaMemcpyAsync(ctx->pool1, static_cast<char*>(ctx->pool) + e, pool_bytes - e,
-                                      cudaMemcpyDeviceToDevice, s), "vr_load_cube: shifted copy");
-                VR_CK(cudaMemsetAsync(static_cast<char*>(ctx->pool1) + pool_bytes - e, 0, e, s),
-                      "vr_load_cube: shifted copy");
-                VR_CK(cudaStreamSynchronize(s), "vr_load_cube: shifted copy");
-            } else {
-                cudaGetLastError();  // not kept: the single-store path serves every render
-                ctx->pool1 = nullptr;
-            }
-        }
-    }
     if (make_tensor_map(ctx)) {
         int cx, cy, cz;
         brick_cell_dims(ctx->dtype, &cx, &cy, &cz);

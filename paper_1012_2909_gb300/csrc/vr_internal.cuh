@@ -182,9 +182,10 @@ struct PixelParams {
 };
 
 // Host-side launchers (defined in the kernel translation units).
-cudaError_t launch_repack(const float* src, long long src_z0, long long src_planes, int bz,
-                          const VolDev& v, vr_dtype dt, void* pool, unsigned int* minmax,
-                          cudaStream_t s);
+// Brick layers [bz0, bz0 + nlayers) of the store (and of its copy shifted by one element,
+// 16-bit stores, when pool1 is given) from the cube planes src_z0 .. at src.
+cudaError_t launch_repack(const float* src, long long src_z0, int bz0, int nlayers, const VolDev& v, vr_dtype dt,
+                          void* pool, void* pool1, unsigned int* minmax, cudaStream_t s);
 // The marcher reads x-neighbour pairs with one load when p.vol.pool1 is set.
 cudaError_t launch_march(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s);
 int march_blocks_per_sm(vr_dtype dt, int mode, bool paired, int block);

@@ -1,8 +1,10 @@
-// Repack of a linear float32 cube (x fastest) into the ghosted brick store:
-// one slab of bricks (fixed bz) per launch, with conversion to the storage type
-// (round to nearest even) and the per-brick minimum / maximum of the stored
-// values (ghost layer included), which bound every trilinear sample taken
-// inside the brick.
+// Repack of a linear float32 cube (x fastest) into the ghosted brick store, with
+// conversion to the storage type (round to nearest even), the store's copy shifted by
+// one element when it is kept, and the per-brick minimum / maximum of the stored
+// values (ghost layer included), which bound every trilinear sample taken inside the
+// brick.
+#include <algorithm>
+
 #include "vr_internal.cuh"
 
 namespace vr {
@@ -27,59 +29,143 @@ template <> __device__ __forceinline__ float widen<__nv_bfloat16>(__nv_bfloat16 
     return __bfloat162float(v);
 }
 
-// grid: (nbx * nby, rows); block: 256.  Block (b, lz) writes plane lz of the
-// slot of brick (b % nbx, b / nbx, bz).
-template <typename T>
-__global__ void __launch_bounds__(256)
-k_repack(const float* __restrict__ src, long long src_z0, int bz, VolDev v, T* __restrict__ pool,
-         unsigned int* __restrict__ minmax, int nbricks) {
-    const int b2 = blockIdx.x;
-    const int bx = b2 % v.nbx, by = b2 / v.nbx;
-    const int lz = blockIdx.y;
+__device__ __forceinline__ unsigned int bits(__half v) { return __half_as_ushort(v); }
+__device__ __forceinline__ unsigned int bits(__nv_bfloat16 v) { return __bfloat16_as_ushort(v); }
+
+__device__ __forceinline__ __half2 pack2(__half a, __half b) { return __halves2half2(a, b); }
+__device__ __forceinline__ __nv_bfloat162 pack2(__nv_bfloat16 a, __nv_bfloat16 b) { return __halves2bfloat162(a, b); }
+
+// Running minimum and maximum of the stored values, a word at a time (NaN ignored, as fminf).
+template <typename T> struct Range {
+    decltype(pack2(T(), T())) mn, mx;
+    __device__ __forceinline__ Range() : mn(pack2(to_store<T>(INFINITY), to_store<T>(INFINITY))),
+                                         mx(pack2(to_store<T>(-INFINITY), to_store<T>(-INFINITY))) {}
+    __device__ __forceinline__ void add(T a, T b) {
+        const auto p = pack2(a, b);
+        mn = __hmin2(mn, p);
+        mx = __hmax2(mx, p);
+    }
+    __device__ __forceinline__ float least() const { return fminf(widen<T>(mn.x), widen<T>(mn.y)); }
+    __device__ __forceinline__ float most() const { return fmaxf(widen<T>(mx.x), widen<T>(mx.y)); }
+};
+template <> struct Range<float> {
+    float mn = INFINITY, mx = -INFINITY;
+    __device__ __forceinline__ void add(float a) {
+        mn = fminf(mn, a);
+        mx = fmaxf(mx, a);
+    }
+    __device__ __forceinline__ float least() const { return mn; }
+    __device__ __forceinline__ float most() const { return mx; }
+};
+
+// grid: (nbx * nby, rows, layers of bricks); block: row_words x `lines` threads, rounded
+// up to whole warps.  Block (b, lz, l) writes plane lz of the slot of brick (b % nbx,
+// b / nbx, bz0 + l), and of its shifted copy.
+//
+// Bound by DRAM: 4 bytes read and sizeof(T) (twice, with the copy) written per voxel.
+// A thread makes one 32-bit word of a row, two 16-bit voxels or one float, and goes
+// down the plane in that column, so its clamped source columns are found once and a
+// word costs few instructions.  Loads and stores of a warp are consecutive words
+// whatever the source's alignment (a row starts one voxel before the brick, so wider
+// loads would never be aligned); kRepackUnroll rows' loads are in flight.  The copy's
+// word (voxels x + 1, x + 2) is made from the same registers and the next lane's, in
+// place of a device-to-device copy at a 2-byte offset afterwards.  REPACK_FIGURES
+constexpr int kRepackUnroll = 4;
+constexpr int kRepackThreads = 288;  // threads of a block, about
+
+template <typename T, bool COPY>
+__global__ void __launch_bounds__(512)
+k_repack(const float* __restrict__ src, long long src_z0, int bz0, VolDev v, T* __restrict__ pool,
+         T* __restrict__ pool1, unsigned int* __restrict__ minmax, int nbricks, int row_words, int lines) {
+    constexpr int VPW = 4 / (int)sizeof(T);  // voxels per word
+    constexpr int U = kRepackUnroll;
+    const int bx = blockIdx.x % v.nbx, by = blockIdx.x / v.nbx, bz = bz0 + blockIdx.z;
+    const int lz = blockIdx.y, lane = threadIdx.x & 31;
     const int bid = (bz * v.nby + by) * v.nbx + bx;
-    const int slot = v.table[bid];
-    T* dst = pool + (long long)slot * v.slot_elems + (long long)lz * v.rows * v.pitch;
+    const long long base = (long long)v.table[bid] * v.slot_elems + (long long)lz * v.rows * v.pitch;
+    unsigned int* dst = reinterpret_cast<unsigned int*>(pool + base);
+    unsigned int* dst1 = COPY ? reinterpret_cast<unsigned int*>(pool1 + base) : nullptr;
     const int gz = min(max(bz * v.B + lz - 1, 0), v.nz - 1);
     const float* plane = src + (long long)(gz - src_z0) * v.ny * v.nx;
-    float mn = INFINITY, mx = -INFINITY;
-    const int n = v.rows * v.pitch;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int ly = i / v.pitch, lx = i - ly * v.pitch;
-        T out = to_store<T>(0.f);
-        if (lx < v.rows) {
-            const int gy = min(max(by * v.B + ly - 1, 0), v.ny - 1);
-            const int gx = min(max(bx * v.B + lx - 1, 0), v.nx - 1);
-            out = to_store<T>(plane[(long long)gy * v.nx + gx]);
-            const float w = widen<T>(out);
-            mn = fminf(mn, w);
-            mx = fmaxf(mx, w);
+    // this thread's line of the block's `lines` rows and its word of the row; a row is a
+    // whole number of voxel words and padding words (rows is even, padding columns are 0)
+    const int line = threadIdx.x / row_words, word = threadIdx.x - line * row_words;
+    const int lx = word * VPW, x0 = bx * v.B - 1 + lx, y0 = by * v.B - 1;
+    const bool mine = line < lines, real = mine && lx < v.rows;
+    const int c0 = min(max(x0, 0), v.nx - 1), c1 = min(max(x0 + 1, 0), v.nx - 1);
+    // lane 31 loads the voxel after its word itself
+    const bool third = COPY && lane == 31 && lx + VPW < v.rows;
+    const int c2 = min(max(x0 + 2, 0), v.nx - 1);
+    Range<T> range;
+    for (int ly0 = line; ly0 - line < v.rows; ly0 += lines * U) {  // the same trips for every lane
+        float f[U][VPW], f2[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float* row = plane + (long long)min(max(y0 + ly0 + u * lines, 0), v.ny - 1) * v.nx;
+            f[u][0] = real ? __ldg(row + c0) : 0.f;
+            if (VPW == 2) f[u][VPW - 1] = real ? __ldg(row + c1) : 0.f;
+            f2[u] = third ? __ldg(row + c2) : 0.f;
         }
-        dst[i] = out;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int ly = ly0 + u * lines;
+            const bool put = mine && ly < v.rows;
+            if constexpr (VPW == 2) {
+                const T a = to_store<T>(f[u][0]), b = to_store<T>(f[u][1]);
+                if (real) range.add(a, b);  // rows past the last repeat it
+                const unsigned int lo = bits(a), hi = bits(b);
+                if (put) dst[ly * row_words + word] = lo | (hi << 16);
+                if (COPY) {
+                    const unsigned int next = __shfl_down_sync(0xffffffffu, lo, 1);
+                    const unsigned int x2 = lane == 31 ? bits(to_store<T>(f2[u])) : next;
+                    if (put) dst1[ly * row_words + word] = hi | (lx + VPW < v.pitch ? x2 << 16 : 0u);
+                }
+            } else {
+                if (real) range.add(f[u][0]);
+                if (put) dst[ly * row_words + word] = __float_as_uint(f[u][0]);
+            }
+        }
     }
+    float mn = range.least(), mx = range.most();
     for (int off = 16; off > 0; off >>= 1) {
         mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     }
-    if ((threadIdx.x & 31) == 0) {
+    if (lane == 0) {
         atomicMin(&minmax[bid], ord_enc(mn));
         atomicMax(&minmax[nbricks + bid], ord_enc(mx));
     }
 }
 
+template <typename T>
+cudaError_t repack_t(const float* src, long long src_z0, int bz0, int nlayers, const VolDev& v, void* pool,
+                     void* pool1, unsigned int* minmax, cudaStream_t s) {
+    const int nbricks = v.nbx * v.nby * v.nbz;
+    const int row_words = v.pitch * (int)sizeof(T) / 4;  // 8 .. 260
+    const int lines = std::max(1, kRepackThreads / row_words);
+    const int block = (row_words * lines + 31) / 32 * 32;
+    for (int l = 0; l < nlayers; l += 65535) {  // a grid's z limit
+        const dim3 grid(v.nbx * v.nby, v.rows, std::min(nlayers - l, 65535));
+        if (sizeof(T) == 2 && pool1)
+            k_repack<T, sizeof(T) == 2><<<grid, block, 0, s>>>(src, src_z0, bz0 + l, v, static_cast<T*>(pool),
+                                                              static_cast<T*>(pool1), minmax, nbricks, row_words,
+                                                              lines);
+        else
+            k_repack<T, false><<<grid, block, 0, s>>>(src, src_z0, bz0 + l, v, static_cast<T*>(pool), nullptr, minmax,
+                                                      nbricks, row_words, lines);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 }  // namespace
 
-cudaError_t launch_repack(const float* src, long long src_z0, long long /*src_planes*/, int bz,
-                          const VolDev& v, vr_dtype dt, void* pool, unsigned int* minmax,
-                          cudaStream_t s) {
-    const dim3 grid(v.nbx * v.nby, v.rows);
-    const int nbricks = v.nbx * v.nby * v.nbz;
-    if (dt == VR_F32)
-        k_repack<float><<<grid, 256, 0, s>>>(src, src_z0, bz, v, static_cast<float*>(pool), minmax, nbricks);
-    else if (dt == VR_F16)
-        k_repack<__half><<<grid, 256, 0, s>>>(src, src_z0, bz, v, static_cast<__half*>(pool), minmax, nbricks);
-    else
-        k_repack<__nv_bfloat16><<<grid, 256, 0, s>>>(src, src_z0, bz, v, static_cast<__nv_bfloat16*>(pool), minmax, nbricks);
-    return cudaGetLastError();
+cudaError_t launch_repack(const float* src, long long src_z0, int bz0, int nlayers, const VolDev& v, vr_dtype dt,
+                          void* pool, void* pool1, unsigned int* minmax, cudaStream_t s) {
+    if (dt == VR_F32) return repack_t<float>(src, src_z0, bz0, nlayers, v, pool, pool1, minmax, s);
+    if (dt == VR_F16) return repack_t<__half>(src, src_z0, bz0, nlayers, v, pool, pool1, minmax, s);
+    return repack_t<__nv_bfloat16>(src, src_z0, bz0, nlayers, v, pool, pool1, minmax, s);
 }
 
 }  // namespace vr
