@@ -734,7 +734,7 @@ __device__ __forceinline__ void build_part_segments(const BrickParams& P, int4 r
 // composited from T = 1 (the warp's lanes all take `iters` steps; steps past the
 // run add nothing: alpha 0 leaves C and T exactly as they are).
 template <typename T, bool CLAMP>
-__device__ __forceinline__ void run_over(const T* __restrict__ tile, const float4* __restrict__ s_tf, const TFDev& tf,
+__device__ __forceinline__ void run_over(const T* __restrict__ tile, const float* __restrict__ s_tf, const TFDev& tf,
                                          const SegRec& s, int n, int k0, int L, int iters, float& C0, float& C1,
                                          float& C2, float& Tr) {
     C0 = C1 = C2 = 0.f;
@@ -745,7 +745,7 @@ __device__ __forceinline__ void run_over(const T* __restrict__ tile, const float
         const float f = fminf((float)k, last);
         const float v = tile_fetch<T, CLAMP, PartGeom<T>::BY>(tile, fmaf(f, s.ex, s.gx), fmaf(f, s.ey, s.gy),
                                                               fmaf(f, s.ez, s.gz));
-        const float4 c = tf_lookup(s_tf, tf.n, tf.vmin, tf.inv_range, v);
+        const float4 c = tf_lookup<kMaxPartTF>(s_tf, tf.n, tf.vmin, tf.inv_range, v);
         const float a = (j < L && k < n) ? c.w : 0.f;
         const float w = Tr * a;
         C0 = fmaf(w, c.x, C0);
@@ -774,7 +774,7 @@ __device__ __forceinline__ float run_max(const T* __restrict__ tile, const SegRe
 // lanes marches one record and its lane 0 folds the result into the record's
 // slot.  A pass never holds two records of one slot.
 template <typename T, int MODE, int G>
-__device__ __forceinline__ void march_part(const BrickParams& P, const T* tile, const float4* s_tf, const TFDev& tf,
+__device__ __forceinline__ void march_part(const BrickParams& P, const T* tile, const float* s_tf, const TFDev& tf,
                                            const SegRec* segs, int nlong, int nshort, int* claim, int lane) {
     constexpr int PER_WARP = 32 / G;
     const int q = lane / G, r = lane % G;
@@ -847,7 +847,7 @@ k_cell_partial(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
     extern __shared__ __align__(128) unsigned char smem[];
     T* tile = reinterpret_cast<T*>(smem);
     SegRec* segs = reinterpret_cast<SegRec*>(smem + PG::STRIDE);
-    float4* s_tf = reinterpret_cast<float4*>(smem + PG::STRIDE + kSegCap * sizeof(SegRec));
+    float* s_tf = reinterpret_cast<float*>(smem + PG::STRIDE + kSegCap * sizeof(SegRec));
     __shared__ __align__(8) uint64_t bar;
     __shared__ CellDesc s_desc[3];
     __shared__ BrickFoot s_foot[3];
@@ -857,8 +857,7 @@ k_cell_partial(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nvalid = *count;
-    if (MODE == VR_COMPOSITE)
-        for (int i = tid; i < tf.n; i += kBrickThreads) s_tf[i] = tf.tab[i];
+    if (MODE == VR_COMPOSITE) fill_table<kMaxPartTF>(s_tf, tf);
     // warp 0: claim the next unit into descriptor slot `slot` (returns the unit)
     auto claim = [&](int slot) {
         int u = 0;
@@ -1006,14 +1005,14 @@ __global__ void k_pixel_setup(const __grid_constant__ PixelParams P) {
 }
 
 __global__ void k_mip_finalize(const __grid_constant__ PixelParams P) {
-    __shared__ float4 s_tf[kMaxTF];
-    for (int i = threadIdx.x; i < P.tf.n; i += blockDim.x) s_tf[i] = P.tf.tab[i];
+    __shared__ float s_tf[4 * kMaxTF];
+    fill_table<kMaxTF>(s_tf, P.tf);
     __syncthreads();
     const int n = P.width * P.height;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float m = ord_dec(P.enc[i]);
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (m > -INFINITY) o = tf_lookup(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, m);
+        if (m > -INFINITY) o = tf_lookup<kMaxTF>(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, m);
         P.out_rgba[i] = o;
         if (P.out_max) P.out_max[i] = m;
     }

@@ -29,8 +29,8 @@ template <typename T, int MODE, bool PAIRED>
 __global__ void __launch_bounds__(256, 2)
 k_march(const __grid_constant__ MarchParams P) {
     constexpr int U = PAIRED ? kMarchUnrollPaired : kMarchUnroll;
-    __shared__ float4 s_tf[kMaxTF];
-    for (int i = threadIdx.x; i < P.tf.n; i += blockDim.x) s_tf[i] = P.tf.tab[i];
+    __shared__ float s_tf[4 * kMaxTF];
+    fill_table<kMaxTF>(s_tf, P.tf);
     __syncthreads();
 
     const int lane = threadIdx.x & 31;
@@ -92,7 +92,7 @@ k_march(const __grid_constant__ MarchParams P) {
                             if (MODE == VR_MIP) {
                                 m_ = fmaxf(m_, v[q]);
                             } else {
-                                const float4 c = tf_lookup(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v[q]);
+                                const float4 c = tf_lookup<kMaxTF>(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v[q]);
                                 const float w = Tr * c.w;
                                 c0 = fmaf(w, c.x, c0);
                                 c1 = fmaf(w, c.y, c1);
@@ -115,7 +115,7 @@ k_march(const __grid_constant__ MarchParams P) {
         const long long pix = ((long long)cam * P.height + py) * P.width + px;
         if (MODE == VR_MIP) {
             float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (m_ > -INFINITY) o = tf_lookup(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, m_);
+            if (m_ > -INFINITY) o = tf_lookup<kMaxTF>(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, m_);
             P.out_rgba[pix] = o;
             if (P.out_max) P.out_max[pix] = m_;
         } else {

@@ -278,8 +278,8 @@ __global__ void k_tile_scan(const __grid_constant__ SortParams P) {
 template <typename T, bool CARRIED>
 __global__ void __launch_bounds__(128)
 k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer_end) {
-    __shared__ float4 s_tf[kMaxTF];
-    for (int i = threadIdx.x; i < P.tf.n; i += blockDim.x) s_tf[i] = P.tf.tab[i];
+    __shared__ float s_tf[4 * kMaxTF];
+    fill_table<kMaxTF>(s_tf, P.tf);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     // the bricks of layers [layer_begin, layer_end) of the ordered list, or an explicit subset
@@ -349,7 +349,7 @@ k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer
                 const float fj = (float)j;
                 const float v = fetch_trilinear<T>(slot, P.vol, fmaf(fj, e[0], g[0]), fmaf(fj, e[1], g[1]),
                                                    fmaf(fj, e[2], g[2]));
-                const float4 c = tf_lookup(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v);
+                const float4 c = tf_lookup<kMaxTF>(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v);
                 const float w = Tr * c.w;
                 C0 = fmaf(w, c.x, C0);
                 C1 = fmaf(w, c.y, C1);
@@ -387,8 +387,8 @@ template <typename T, bool PAIRED>
 __global__ void __launch_bounds__(256, 2)
 k_march_layered(const __grid_constant__ MarchParams P) {
     constexpr int U = PAIRED ? kLayeredUnrollPaired : kLayeredUnroll;
-    __shared__ float4 s_tf[kMaxTF];
-    for (int i = threadIdx.x; i < P.tf.n; i += blockDim.x) s_tf[i] = P.tf.tab[i];
+    __shared__ float s_tf[4 * kMaxTF];
+    fill_table<kMaxTF>(s_tf, P.tf);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int tiles_per_cam = P.tiles_x * P.tiles_y;
@@ -472,7 +472,7 @@ k_march_layered(const __grid_constant__ MarchParams P) {
 #pragma unroll
                         for (int q = 0; q < U; ++q) {
                             if (i + q >= n) break;
-                            const float4 t = tf_lookup(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v[q]);
+                            const float4 t = tf_lookup<kMaxTF>(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v[q]);
                             const float w = Tr * t.w;
                             C0 = fmaf(w, t.x, C0);
                             C1 = fmaf(w, t.y, C1);
