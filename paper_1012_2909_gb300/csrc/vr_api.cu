@@ -1661,6 +1661,11 @@ vr_status vr_render_backward(vr_ctx* ctx, vr_mode mode, const float* dL_dimg, fl
     P.tiles_y = (P.height + kTileH - 1) / kTileH;
     split(ctx->opt.step, P.step_hi, P.step_lo);
     P.ert = (float)ctx->opt.ert;
+    P.tf_unit = 1;
+    for (const float4& t : ctx->tf) {
+        if (!(t.w >= 0.f && t.w <= 1.f)) P.tf_unit = 0;
+        P.tf_cmax = std::max(P.tf_cmax, std::max(std::fabs(t.x), std::max(std::fabs(t.y), std::fabs(t.z))));
+    }
     P.dvol = dL_dvol;
     P.status = ctx->status_dev;
     const long long img = (long long)P.width * P.height;

@@ -123,7 +123,8 @@ struct AdjParams {
     int tiles_x, tiles_y;
     float step_hi, step_lo;  // the sample spacing as a float-float pair
     float ert;
-    int pad2;
+    int tf_unit;          // every opacity of the table is in [0, 1]
+    float tf_cmax;        // its largest colour magnitude
     const float4* dimg;   // dL/dI of camera 0 of this launch
     float* dvol;          // dL/dvoxel, linear x-fastest (may be null)
     float* tf_partials;   // per-block table partials of this launch (grid x ntf x 4)
