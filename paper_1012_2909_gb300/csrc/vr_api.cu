@@ -804,9 +804,30 @@ vr_status ensure_pixel_scratch(vr_ctx* ctx, long long npix) {
     return VR_OK;
 }
 
+// The set-up of W x H views (cameras, outputs and ncams > 1 are the caller's to fill in).
+SetupParams setup_params(const vr_ctx* ctx, int W, int H) {
+    SetupParams p;
+    std::memset(&p, 0, sizeof(p));
+    p.vol = vol_dev(ctx);
+    split(ctx->opt.step, p.step_hi, p.step_lo);
+    p.ncams = 1;
+    p.width = W;
+    p.height = H;
+    p.krange = ctx->krange;
+    p.pixdir = ctx->pixdir;
+    return p;
+}
+
+FinalizeParams finalize_params(const vr_ctx* ctx) {
+    FinalizeParams p;
+    std::memset(&p, 0, sizeof(p));
+    p.tf = tf_dev(ctx);
+    return p;
+}
+
 // MIP through the brick pass, up to kMaxLaunchCams cameras per pass over the
-// cube: pixel set-up per camera (sample ranges, running maxima), one staged
-// brick pass for the batch, transfer-function finalisation per camera.
+// cube: pixel set-up (sample ranges, running maxima, the pass's counters), one staged
+// brick pass, transfer-function finalisation, a launch each for the batch.
 vr_status render_brick_mip(vr_ctx* ctx, float* out_rgba, float* out_max, cudaStream_t s) {
     const int W = ctx->cams[0].width, H = ctx->cams[0].height;
     const long long img = (long long)W * H;
@@ -816,13 +837,8 @@ vr_status render_brick_mip(vr_ctx* ctx, float* out_rgba, float* out_max, cudaStr
     const int per = (int)std::min<long long>(std::min(ncams, kMaxLaunchCams), std::max(1LL, INT_MAX / img));
     vr_status st = ensure_pixel_scratch(ctx, img * per);
     if (st != VR_OK) return st;
-    PixelParams pp;
-    std::memset(&pp, 0, sizeof(pp));
-    pp.vol = vol_dev(ctx);
-    pp.tf = tf_dev(ctx);
-    split(ctx->opt.step, pp.step_hi, pp.step_lo);
-    pp.width = W;
-    pp.height = H;
+    SetupParams pp = setup_params(ctx, W, H);
+    FinalizeParams fp = finalize_params(ctx);
     BrickParams bp;
     std::memset(&bp, 0, sizeof(bp));
     bp.vol = pp.vol;
@@ -846,26 +862,24 @@ vr_status render_brick_mip(vr_ctx* ctx, float* out_rgba, float* out_max, cudaStr
         for (int i = 0; i < nb; ++i) {
             if (!cam_ff(ctx->cams[(size_t)(c0 + i)], bp.cams[i]))
                 return fail(ctx, VR_ERR_INVALID_ARG, "vr_render: camera basis is singular");
-            pp.cam = ray_cam(ctx->cams[(size_t)(c0 + i)]);
-            pp.krange = ctx->krange + (long long)i * img;
-            pp.pixdir = ctx->pixdir + 2 * (long long)i * img;
-            pp.enc = enc + (long long)i * img;
-            VR_CK(launch_pixel_setup(pp, s), "vr_render: pixel set-up");
+            pp.cams[i] = bp.cams[i];
         }
         bp.out_enc = enc;
         bp.work = ctx->work + kMaxLaunchCams + (c0 / per) % 4096;
-        VR_CK(cudaMemsetAsync(bp.work, 0, sizeof(int), s), "vr_render: scheduler reset");
+        pp.ncams = nb;
+        pp.enc = enc;
+        pp.zero[0] = bp.work;
+        pp.zero[1] = static_cast<int*>(ctx->cells);
+        VR_CK(launch_pixel_setup(pp, s), "vr_render: pixel set-up");
         if (c0 == 0 && ctx->ev_start) VR_CK(cudaEventRecord(ctx->ev_start, s), "vr_render: profiling event");
         VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, grid, ctx->cells, s, ctx->tune.group),
               "vr_render: brick pass");
         if (c0 + nb >= ncams && ctx->ev_stop) VR_CK(cudaEventRecord(ctx->ev_stop, s), "vr_render: profiling event");
-        for (int i = 0; i < nb; ++i) {
-            pp.cam = ray_cam(ctx->cams[(size_t)(c0 + i)]);
-            pp.enc = enc + (long long)i * img;
-            pp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)(c0 + i) * img;
-            pp.out_max = out_max ? out_max + (long long)(c0 + i) * img : nullptr;
-            VR_CK(launch_mip_finalize(pp, s), "vr_render: finalise");
-        }
+        fp.npix = (long long)nb * img;
+        fp.enc = enc;
+        fp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)c0 * img;
+        fp.out_max = out_max ? out_max + (long long)c0 * img : nullptr;
+        VR_CK(launch_mip_finalize(fp, s), "vr_render: finalise");
     }
     return VR_OK;
 }
@@ -976,16 +990,7 @@ vr_status render_sortlast_composite(vr_ctx* ctx, float* out_rgba, cudaStream_t s
     sp.order = ctx->order;
     sp.tile_start = ctx->tile_start;
     sp.partial_used = ctx->partial_used;
-    PixelParams pp;
-    std::memset(&pp, 0, sizeof(pp));
-    pp.vol = sp.vol;
-    pp.tf = sp.tf;
-    split(ctx->opt.step, pp.step_hi, pp.step_lo);
-    pp.width = W;
-    pp.height = H;
-    pp.krange = ctx->krange;
-    pp.pixdir = ctx->pixdir;
-    pp.enc = ctx->enc;
+    SetupParams pp = setup_params(ctx, W, H);
     const int grid = ctx->num_sms * 8;
     for (size_t ci = 0; ci < ctx->cams.size(); ++ci) {
         const CamDev& cd = ctx->cams[ci];
@@ -1005,7 +1010,7 @@ vr_status render_sortlast_composite(vr_ctx* ctx, float* out_rgba, cudaStream_t s
         sp.layer_start = ctx->layer_buf + (L + 1);
         sp.layer_fill = ctx->layer_buf + 2 * (L + 1);
         sp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)ci * img;
-        pp.cam = ray_cam(cd);
+        pp.cams[0] = sp.cam;
         VR_CK(launch_pixel_setup(pp, s), "vr_render: pixel set-up");
         VR_CK(cudaMemsetAsync(sp.layer_count, 0, sizeof(int) * (size_t)L, s), "vr_render: reset");
         VR_CK(cudaMemsetAsync(sp.partial_used, 0, sizeof(unsigned long long), s), "vr_render: reset");
@@ -1213,15 +1218,9 @@ vr_status render_ooc(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
     sp.ert = (float)ctx->opt.ert;
     sp.krange = ctx->krange;
     sp.state = ctx->state;
-    PixelParams pp;
-    std::memset(&pp, 0, sizeof(pp));
-    pp.vol = sp.vol;
-    pp.tf = sp.tf;
-    split(ctx->opt.step, pp.step_hi, pp.step_lo);
-    pp.width = W;
-    pp.height = H;
-    pp.krange = ctx->krange;
-    pp.pixdir = ctx->pixdir;
+    SetupParams pp = setup_params(ctx, W, H);
+    FinalizeParams fp = finalize_params(ctx);
+    fp.npix = img;
     BrickParams bp;
     std::memset(&bp, 0, sizeof(bp));
     bp.vol = sp.vol;
@@ -1244,10 +1243,11 @@ vr_status render_ooc(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
         const CamDev& cd = ctx->cams[ci];
         st = ooc_footprints(ctx, cd, sp, order, layer_start, foot, s);
         if (st != VR_OK) return st;
-        pp.cam = ray_cam(cd);
-        pp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)ci * img;
-        pp.out_max = out_max ? out_max + (long long)ci * img : nullptr;
-        pp.enc = (mode == VR_MIP && out_max) ? reinterpret_cast<unsigned int*>(pp.out_max) : ctx->enc;
+        pp.cams[0] = ray_cam(cd);
+        fp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)ci * img;
+        fp.out_max = out_max ? out_max + (long long)ci * img : nullptr;
+        pp.enc = (mode == VR_MIP && out_max) ? reinterpret_cast<unsigned int*>(fp.out_max) : ctx->enc;
+        fp.enc = pp.enc;
         VR_CK(launch_pixel_setup(pp, s), "out of core: pixel set-up");
         if (mode == VR_MIP) {
             if (!cam_ff(cd, bp.cams[0])) return fail(ctx, VR_ERR_INVALID_ARG, "vr_render: camera basis is singular");
@@ -1261,14 +1261,15 @@ vr_status render_ooc(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
                 bp.nlist = n;
                 bp.work = ctx->work;
                 VR_CK(cudaMemsetAsync(bp.work, 0, sizeof(int), s), "out of core: scheduler reset");
+                VR_CK(cudaMemsetAsync(ctx->cells, 0, sizeof(int), s), "out of core: cell count reset");
                 VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s, ctx->tune.group),
                       "out of core: brick pass");
             }
-            VR_CK(launch_mip_finalize(pp, s), "out of core: finalise");
+            VR_CK(launch_mip_finalize(fp, s), "out of core: finalise");
             continue;
         }
         // composite: layer by layer, skipping bricks behind terminated pixels
-        sp.out_rgba = pp.out_rgba;
+        sp.out_rgba = fp.out_rgba;
         VR_CK(launch_state_init(sp, s), "out of core: state init");
         const int L = sp.max_layers;
         for (int l = 0; l < L; ++l) {
@@ -1363,14 +1364,15 @@ vr_status brick_mip_with_scratch(vr_ctx* ctx, float* out_rgba, float* out_max, c
     const int W = ctx->cams[0].width, H = ctx->cams[0].height;
     const long long img = (long long)W * H;
     VR_CK(cudaGetLastError(), "pending CUDA error");
-    PixelParams pp;
-    std::memset(&pp, 0, sizeof(pp));
-    pp.vol = vol_dev(ctx);
-    pp.tf = tf_dev(ctx);
-    split(ctx->opt.step, pp.step_hi, pp.step_lo);
-    pp.width = W;
-    pp.height = H;
+    SetupParams pp = setup_params(ctx, W, H);
     pp.krange = krange;
+    pp.pixdir = nullptr;
+    pp.zero[0] = work;
+    pp.zero[1] = static_cast<int*>(ctx->cells);
+    pp.enc = enc;
+    FinalizeParams fp = finalize_params(ctx);
+    fp.npix = img;
+    fp.enc = enc;
     BrickParams bp;
     std::memset(&bp, 0, sizeof(bp));
     bp.vol = pp.vol;
@@ -1391,16 +1393,14 @@ vr_status brick_mip_with_scratch(vr_ctx* ctx, float* out_rgba, float* out_max, c
     for (int i = 0; i < ncams; ++i) {
         if (!cam_ff(ctx->cams[(size_t)i], bp.cams[0]))
             return fail(ctx, VR_ERR_INVALID_ARG, "camera basis is singular");
-        pp.cam = ray_cam(ctx->cams[(size_t)i]);
-        pp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)i * img;
-        pp.out_max = out_max ? out_max + (long long)i * img : nullptr;
-        pp.enc = enc;
+        pp.cams[0] = bp.cams[0];
+        fp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)i * img;
+        fp.out_max = out_max ? out_max + (long long)i * img : nullptr;
         bp.out_enc = enc;
-        VR_CK(cudaMemsetAsync(work, 0, sizeof(int), s), "scheduler reset");
         VR_CK(launch_pixel_setup(pp, s), "pixel set-up");
         VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s, ctx->tune.group),
               "brick pass");
-        VR_CK(launch_mip_finalize(pp, s), "finalise");
+        VR_CK(launch_mip_finalize(fp, s), "finalise");
     }
     return VR_OK;
 }
@@ -1862,17 +1862,8 @@ vr_status vr_sortlast_partials(vr_ctx* ctx, vr_mode mode, const int32_t* bricks,
     sp.ert = 2.0f;
     sp.mode = mode;
     sp.krange = ctx->krange;
-    PixelParams pp;
-    std::memset(&pp, 0, sizeof(pp));
-    pp.vol = sp.vol;
-    pp.tf = sp.tf;
-    split(ctx->opt.step, pp.step_hi, pp.step_lo);
-    pp.width = W;
-    pp.height = H;
-    pp.krange = ctx->krange;
-    pp.pixdir = ctx->pixdir;
-    pp.enc = ctx->enc;
-    pp.cam = ray_cam(cd);
+    SetupParams pp = setup_params(ctx, W, H);
+    pp.cams[0] = ray_cam(cd);
     VR_CK(launch_pixel_setup(pp, s), "vr_sortlast_partials: pixel set-up");
     std::vector<int> order, layer_start;
     std::vector<BrickFoot> all;

@@ -990,26 +990,32 @@ cudaError_t cell_partials_t(const void* tmap, const BrickParams& p0, const TFDev
     return cudaSuccess;
 }
 
-__global__ void k_pixel_setup(const __grid_constant__ PixelParams P) {
-    const int n = P.width * P.height;
+// Set-up and finalisation of all the cameras of a brick pass in one launch each (grid y:
+// the camera).  A launch per camera, with the 16 KB table among its parameters, and two
+// memsets for the counters that the set-up now clears, cost a small view of two cameras
+// more than its kernels: SETUP_FIGURES
+__global__ void __launch_bounds__(256) k_pixel_setup(const __grid_constant__ SetupParams P) {
+    const int n = P.width * P.height, cam = blockIdx.y;
+    if (blockIdx.x == 0 && cam == 0 && threadIdx.x < 2 && P.zero[threadIdx.x]) *P.zero[threadIdx.x] = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         Ray r;
-        const bool hit = make_ray(P.cam, i % P.width, i / P.width, P.vol, ff{P.step_hi, P.step_lo}, r);
-        P.krange[i] = make_int2(r.k0, r.k1);
-        P.enc[i] = ord_enc(-INFINITY);
-        if (hit && P.pixdir && P.cam.type == 1) {  // read only for pixels with samples
-            P.pixdir[2 * (long long)i] = make_float4(r.e[0].hi, r.e[1].hi, r.e[2].hi, r.e[0].lo);
-            P.pixdir[2 * (long long)i + 1] = make_float4(r.e[1].lo, r.e[2].lo, 0.f, 0.f);
+        const bool hit = make_ray(P.cams[cam], i % P.width, i / P.width, P.vol, ff{P.step_hi, P.step_lo}, r);
+        const long long o = (long long)cam * n + i;
+        P.krange[o] = make_int2(r.k0, r.k1);
+        if (P.enc) P.enc[o] = ord_enc(-INFINITY);
+        if (hit && P.pixdir && P.cams[cam].type == 1) {  // read only for pixels with samples
+            P.pixdir[2 * o] = make_float4(r.e[0].hi, r.e[1].hi, r.e[2].hi, r.e[0].lo);
+            P.pixdir[2 * o + 1] = make_float4(r.e[1].lo, r.e[2].lo, 0.f, 0.f);
         }
     }
 }
 
-__global__ void k_mip_finalize(const __grid_constant__ PixelParams P) {
+__global__ void __launch_bounds__(256) k_mip_finalize(const __grid_constant__ FinalizeParams P) {
     __shared__ float s_tf[4 * kMaxTF];
     fill_table<kMaxTF>(s_tf, P.tf);
     __syncthreads();
-    const int n = P.width * P.height;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P.npix;
+         i += (long long)gridDim.x * blockDim.x) {
         const float m = ord_dec(P.enc[i]);
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
         if (m > -INFINITY) o = tf_lookup<kMaxTF>(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, m);
@@ -1041,8 +1047,6 @@ cudaError_t launch_t(const void* tmap, const BrickParams& p, int grid, void* cel
     CellDesc* list = reinterpret_cast<CellDesc*>(static_cast<char*>(cells) + 256);
     int* count = static_cast<int*>(cells);
     const int nunits = (p.brick_list ? p.nlist : p.nbricks) * p.ncells_x * p.ncells_y * p.ncells_z;
-    cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
     k_cell_list<T><<<std::min((nunits + 255) / 256, 4096), 256, 0, s>>>(p, list, count);
     if (group == 4) return launch_brick_g<T, 4>(tmap, p, grid, list, count, s);
     if (group == 16) return launch_brick_g<T, 16>(tmap, p, grid, list, count, s);
@@ -1101,16 +1105,15 @@ cudaError_t launch_cell_partials(const void* tmap, const BrickParams& p, const T
     return cell_partials_t<__nv_bfloat16>(tmap, p, tf, mode, npartial, npass, grid, cells, s, group);
 }
 
-cudaError_t launch_pixel_setup(const PixelParams& p, cudaStream_t s) {
+cudaError_t launch_pixel_setup(const SetupParams& p, cudaStream_t s) {
     const int n = p.width * p.height;
-    const int grid = std::min((n + 255) / 256, 152 * 8);
+    const dim3 grid(std::max(1, std::min((n + 255) / 256, 152 * 8 / p.ncams)), p.ncams);
     k_pixel_setup<<<grid, 256, 0, s>>>(p);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mip_finalize(const PixelParams& p, cudaStream_t s) {
-    const int n = p.width * p.height;
-    const int grid = std::min((n + 255) / 256, 152 * 8);
+cudaError_t launch_mip_finalize(const FinalizeParams& p, cudaStream_t s) {
+    const int grid = (int)std::min<long long>((p.npix + 255) / 256, 152 * 8);
     k_mip_finalize<<<grid, 256, 0, s>>>(p);
     return cudaGetLastError();
 }

@@ -168,18 +168,26 @@ struct SortParams {
                                       // band image (fold_rows = 0: the whole image)
 };
 
-// Per-pixel set-up and finalisation around the brick pass.
-struct PixelParams {
+// Per-pixel set-up before the brick passes: up to kMaxLaunchCams cameras of one size,
+// per-pixel arrays camera-major.
+struct SetupParams {
     VolDev vol;
-    TFDev tf;
-    CamFF cam;
+    CamFF cams[kMaxLaunchCams];
     float step_hi, step_lo;
-    int width, height;
+    int ncams, width, height;
+    int* zero[2];       // optional counters of the passes that follow, set to 0
     int2* krange;
-    float4* pixdir;  // optional: per-pixel float-float step vector (see BrickParams)
-    unsigned int* enc;
+    float4* pixdir;     // optional: per-pixel float-float step vector (see BrickParams)
+    unsigned int* enc;  // optional: running maxima, set to -inf
+};
+
+// Finalisation after the brick pass: npix maxima (of any number of images) to colours.
+struct FinalizeParams {
+    TFDev tf;
+    long long npix;
+    const unsigned int* enc;
     float4* out_rgba;
-    float* out_max;
+    float* out_max;  // may be null, or enc itself
 };
 
 // Host-side launchers (defined in the kernel translation units).
@@ -194,10 +202,11 @@ int march_blocks_per_sm(vr_dtype dt, int mode, bool paired, int block);
 // positioned brick by brick as in launch_brick_partial.
 cudaError_t launch_march_layered(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s);
 int layered_blocks_per_sm(vr_dtype dt, bool paired, int block);
-cudaError_t launch_pixel_setup(const PixelParams& p, cudaStream_t s);
-cudaError_t launch_mip_finalize(const PixelParams& p, cudaStream_t s);
+cudaError_t launch_pixel_setup(const SetupParams& p, cudaStream_t s);
+cudaError_t launch_mip_finalize(const FinalizeParams& p, cudaStream_t s);
 // `cells` is per-context scratch of brick_cells_bytes(units) bytes (a counter and the
-// per-view list of cells with work); the brick kernel's work counter is p.work.
+// per-view list of cells with work); the brick kernel's work counter is p.work.  Both
+// counters must be 0 (SetupParams::zero, or memsets).
 cudaError_t launch_brick_mip(const void* tmap, const BrickParams& p, vr_dtype dt, int grid, void* cells,
                              cudaStream_t s, int group = 8);
 size_t brick_cells_bytes(long long nunits);
