@@ -675,8 +675,7 @@ k_brick_mip(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ Br
 // MIP).  The brick's cells split those samples by the same face-crossing rule,
 // so the partial is the front-to-back fold of the pixel's cell segments.  Each
 // visibility pass stages the cells of one local key (k_cell_list), marches each
-// segment with G lanes on contiguous runs of samples, joins the runs in ray
-// order, and folds the segment into the brick's slot: C += T C_seg, T *= T_seg
+// segment with G lanes on consecutive samples, and folds the segment into the brick's slot: C += T C_seg, T *= T_seg
 // (or the maximum).  Slots start as the empty image (0, 0, 0, 1), or -inf.
 
 // Staged box without the spare row (the partial pass also holds the table).
@@ -730,28 +729,43 @@ __device__ __forceinline__ void build_part_segments(const BrickParams& P, int4 r
     }
 }
 
-// One lane's contiguous run of a segment, samples [k0, k0 + L) clipped to n,
-// composited from T = 1 (the warp's lanes all take `iters` steps; steps past the
-// run add nothing: alpha 0 leaves C and T exactly as they are).
-template <typename T, bool CLAMP>
+// A segment's "over" from T = 1 by a group of G lanes, a step on G consecutive samples, a
+// lane each.  The transmittance before each sample is the carried one times a prefix
+// product over the group; every lane adds up the colour of its own samples.  Returns each
+// lane's colour (their sum is the segment's) and the segment's transmittance.  (The warp's
+// lanes all take `iters` steps; samples past the end add nothing: opacity 0.)
+//
+// Bound by the shared-memory pipe (l1tex 91 % busy with contiguous runs of samples a
+// lane, joined once at the end): lanes half a voxel apart share words of the tile, lanes
+// some 4 voxels apart fall on random banks, and that saves more wavefronts than the five
+// shuffles a step take.  Survey frame: 4.59 -> 4.24 ms; two consecutive samples a lane
+// and step 4.36, four 4.87 ms.
+template <typename T, int G, bool CLAMP>
 __device__ __forceinline__ void run_over(const T* __restrict__ tile, const float* __restrict__ s_tf, const TFDev& tf,
-                                         const SegRec& s, int n, int k0, int L, int iters, float& C0, float& C1,
-                                         float& C2, float& Tr) {
+                                         const SegRec& s, int n, int r, int iters, float& C0, float& C1, float& C2,
+                                         float& Tr) {
     C0 = C1 = C2 = 0.f;
     Tr = 1.f;
     const float last = (float)(n - 1);
     for (int j = 0; j < iters; ++j) {
-        const int k = k0 + j;
+        const int k = j * G + r;
         const float f = fminf((float)k, last);
         const float v = tile_fetch<T, CLAMP, PartGeom<T>::BY>(tile, fmaf(f, s.ex, s.gx), fmaf(f, s.ey, s.gy),
                                                               fmaf(f, s.ez, s.gz));
         const float4 c = tf_lookup<kMaxPartTF>(s_tf, tf.n, tf.vmin, tf.inv_range, v);
-        const float a = (j < L && k < n) ? c.w : 0.f;
-        const float w = Tr * a;
+        const float a = k < n ? c.w : 0.f;
+        float incl = 1.f - a;
+#pragma unroll
+        for (int d = 1; d < G; d <<= 1) {
+            const float t = __shfl_up_sync(0xffffffffu, incl, d, G);
+            if (r >= d) incl *= t;
+        }
+        const float excl = __shfl_up_sync(0xffffffffu, incl, 1, G);
+        const float w = (r == 0 ? Tr : Tr * excl) * a;
+        Tr *= __shfl_sync(0xffffffffu, incl, G - 1, G);
         C0 = fmaf(w, c.x, C0);
         C1 = fmaf(w, c.y, C1);
         C2 = fmaf(w, c.z, C2);
-        Tr = Tr * (1.f - a);
     }
 }
 
@@ -801,30 +815,21 @@ __device__ __forceinline__ void march_part(const BrickParams& P, const T* tile, 
                 d->x = fmaxf(d->x, m);
             }
         } else {
-            const int L = (n + G - 1) / G;  // samples per lane: lane r takes [r L, r L + L)
-            const int iters = (int)__reduce_max_sync(0xffffffffu, (unsigned int)L);
+            const int iters = (int)__reduce_max_sync(0xffffffffu, (unsigned int)((n + G - 1) / G));
             // the slot's state, read before the march (no other record of this pass
             // writes it), so that its latency hides behind the samples
             float4 p = make_float4(0.f, 0.f, 0.f, 1.f);
             if (writer) p = __ldcg(P.partial + s.pix);
             float C0, C1, C2, Tr;
             if (clamp)
-                run_over<T, true>(tile, s_tf, tf, s, n, r * L, L, iters, C0, C1, C2, Tr);
+                run_over<T, G, true>(tile, s_tf, tf, s, n, r, iters, C0, C1, C2, Tr);
             else
-                run_over<T, false>(tile, s_tf, tf, s, n, r * L, L, iters, C0, C1, C2, Tr);
-            // join the runs in ray order: (C, T) of lanes r and r + d, then r and r + 2d, ...
+                run_over<T, G, false>(tile, s_tf, tf, s, n, r, iters, C0, C1, C2, Tr);
 #pragma unroll
-            for (int d = 1; d < G; d <<= 1) {
-                const float p0 = __shfl_down_sync(0xffffffffu, C0, d, G);
-                const float p1 = __shfl_down_sync(0xffffffffu, C1, d, G);
-                const float p2 = __shfl_down_sync(0xffffffffu, C2, d, G);
-                const float pT = __shfl_down_sync(0xffffffffu, Tr, d, G);
-                if ((r & (2 * d - 1)) == 0) {
-                    C0 = fmaf(Tr, p0, C0);
-                    C1 = fmaf(Tr, p1, C1);
-                    C2 = fmaf(Tr, p2, C2);
-                    Tr *= pT;
-                }
+            for (int d = G / 2; d > 0; d >>= 1) {
+                C0 += __shfl_xor_sync(0xffffffffu, C0, d);
+                C1 += __shfl_xor_sync(0xffffffffu, C1, d);
+                C2 += __shfl_xor_sync(0xffffffffu, C2, d);
             }
             if (writer) {
                 p.x = fmaf(p.w, C0, p.x);
@@ -993,7 +998,7 @@ cudaError_t cell_partials_t(const void* tmap, const BrickParams& p0, const TFDev
 // Set-up and finalisation of all the cameras of a brick pass in one launch each (grid y:
 // the camera).  A launch per camera, with the 16 KB table among its parameters, and two
 // memsets for the counters that the set-up now clears, cost a small view of two cameras
-// more than its kernels: SETUP_FIGURES
+// more than its kernels (96 x 80 x 72, two views of 64 x 48: 55.7 -> 44.9 us, host-bound).
 __global__ void __launch_bounds__(256) k_pixel_setup(const __grid_constant__ SetupParams P) {
     const int n = P.width * P.height, cam = blockIdx.y;
     if (blockIdx.x == 0 && cam == 0 && threadIdx.x < 2 && P.zero[threadIdx.x]) *P.zero[threadIdx.x] = 0;
