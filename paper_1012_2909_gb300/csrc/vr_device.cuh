@@ -286,10 +286,8 @@ __device__ __forceinline__ float fetch_trilinear_pair(const T* __restrict__ slot
 // coordinate q = q0 + j e stays below 1 + kAnchorSpan |e| in magnitude: the
 // position keeps about 2^-24 of that magnitude, not of the brick edge.
 struct Anchor {
-    float qx, qy, qz;     // remainder at the anchor sample
-    float lox, loy, loz;  // clamp of q to the slot: [-G, B + 0.999 - G]
-    float hix, hiy, hiz;
-    int base;             // element offset of voxel G in the slot
+    float qx, qy, qz;  // remainder at the anchor sample
+    int base;          // element offset of voxel G in the slot
 };
 
 constexpr int kAnchorSpan = 12;  // samples per sub-anchor
@@ -297,7 +295,7 @@ constexpr int kAnchorSpan = 12;  // samples per sub-anchor
 __device__ __forceinline__ Anchor anchor_at(const Ray& r, int k, const VolDev& v, const Seg& s) {
     const ff kk = ff_of_int(k);
     const float org[3] = {s.ox, s.oy, s.oz};
-    float q[3], lo[3], hi[3];
+    float q[3];
     int G[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -307,39 +305,60 @@ __device__ __forceinline__ Anchor anchor_at(const Ray& r, int k, const VolDev& v
         const float g0 = floorf(gh);
         q[a] = __fadd_rn(__fsub_rn(gh, g0), p.lo);
         G[a] = (int)g0;
-        lo[a] = -g0;
-        hi[a] = __fadd_rn((float)v.B - g0, 0.999f);
     }
     Anchor A;
     A.qx = q[0];
     A.qy = q[1];
     A.qz = q[2];
-    A.lox = lo[0];
-    A.loy = lo[1];
-    A.loz = lo[2];
-    A.hix = hi[0];
-    A.hiy = hi[1];
-    A.hiz = hi[2];
     A.base = (G[2] * v.rows + G[1]) * v.pitch + G[0];
     return A;
 }
 
+// Row pitch and slab of a slot in elements: constants for the default brick edge (BR =
+// 128), so that the eight corners are one address and immediate offsets, else (BR = 0)
+// read from the volume.
+template <typename T, int BR> struct SlotGeom {
+    static constexpr int VEC = 16 / (int)sizeof(T), ROWS = BR + 2, PITCH = (ROWS + VEC - 1) / VEC * VEC;
+    __device__ __forceinline__ static int pitch(const VolDev& v) { return BR ? PITCH : v.pitch; }
+    __device__ __forceinline__ static int slab(const VolDev& v) { return BR ? ROWS * PITCH : v.rows * v.pitch; }
+    // last lower corner whose upper corner lies in the slot
+    __device__ __forceinline__ static unsigned int last(const VolDev& v) {
+        const int rows = BR ? ROWS : v.rows;
+        return (unsigned int)(rows * slab(v) - slab(v) - pitch(v) - 2);
+    }
+};
+
+// Element offset of the lower corner floor(q) from the anchor's, and q's fractions.  A
+// segment's samples lie inside the slot (seg_begin cuts it half a voxel before the ghost
+// layer ends, and the anchors keep them there to 1e-6 voxel), so q is not clamped; the
+// offset is, to the slot, so that nothing outside it can be read.
+template <typename T, int BR>
+__device__ __forceinline__ int near_offset(const VolDev& v, const Anchor& A, float qx, float qy, float qz, float& fx,
+                                           float& fy, float& fz) {
+    const float x0 = floorf(qx), y0 = floorf(qy), z0 = floorf(qz);
+    fx = qx - x0;
+    fy = qy - y0;
+    fz = qz - z0;
+    int o;
+    if (BR)  // exact: the whole slot is below 2^24 elements
+        o = (int)fmaf(fmaf(z0, (float)(BR + 2), y0), (float)SlotGeom<T, BR>::PITCH, x0);
+    else
+        o = ((int)z0 * v.rows + (int)y0) * v.pitch + (int)x0;
+    return (int)min((unsigned int)(A.base + o), SlotGeom<T, BR>::last(v));
+}
+
 // fetch_trilinear at slot coordinate G + q for the anchor's G: the same lerps on the
 // same voxels, with the corner index split as base(G) + index(floor q).
-template <typename T>
+template <typename T, int BR>
 __device__ __forceinline__ float fetch_near(const T* __restrict__ slot, const VolDev& v, const Anchor& A,
                                             float qx, float qy, float qz) {
-    qx = fminf(fmaxf(qx, A.lox), A.hix);
-    qy = fminf(fmaxf(qy, A.loy), A.hiy);
-    qz = fminf(fmaxf(qz, A.loz), A.hiz);
-    const float fx0 = floorf(qx), fy0 = floorf(qy), fz0 = floorf(qz);
-    const float fx = qx - fx0, fy = qy - fy0, fz = qz - fz0;
-    const int slab = v.rows * v.pitch;
-    const T* p = slot + A.base + ((int)fz0 * v.rows + (int)fy0) * v.pitch + (int)fx0;
+    float fx, fy, fz;
+    const T* p = slot + near_offset<T, BR>(v, A, qx, qy, qz, fx, fy, fz);
+    const int pitch = SlotGeom<T, BR>::pitch(v), slab = SlotGeom<T, BR>::slab(v);
     const float c000 = ld_voxel(p), c100 = ld_voxel(p + 1);
-    const float c010 = ld_voxel(p + v.pitch), c110 = ld_voxel(p + v.pitch + 1);
+    const float c010 = ld_voxel(p + pitch), c110 = ld_voxel(p + pitch + 1);
     const float c001 = ld_voxel(p + slab), c101 = ld_voxel(p + slab + 1);
-    const float c011 = ld_voxel(p + slab + v.pitch), c111 = ld_voxel(p + slab + v.pitch + 1);
+    const float c011 = ld_voxel(p + slab + pitch), c111 = ld_voxel(p + slab + pitch + 1);
     const float a0 = fmaf(fx, c100 - c000, c000), a1 = fmaf(fx, c110 - c010, c010);
     const float a2 = fmaf(fx, c101 - c001, c001), a3 = fmaf(fx, c111 - c011, c011);
     const float b0 = fmaf(fy, a1 - a0, a0), b1 = fmaf(fy, a3 - a2, a2);
@@ -347,20 +366,15 @@ __device__ __forceinline__ float fetch_near(const T* __restrict__ slot, const Vo
 }
 
 // fetch_trilinear_pair at slot coordinate G + q for the anchor's G (see fetch_near).
-template <typename T>
+template <typename T, int BR>
 __device__ __forceinline__ float fetch_near_pair(const T* __restrict__ slot, const T* __restrict__ slot1,
                                                  const VolDev& v, const Anchor& A, float qx, float qy, float qz) {
-    qx = fminf(fmaxf(qx, A.lox), A.hix);
-    qy = fminf(fmaxf(qy, A.loy), A.hiy);
-    qz = fminf(fmaxf(qz, A.loz), A.hiz);
-    const float fx0 = floorf(qx), fy0 = floorf(qy), fz0 = floorf(qz);
-    const float fx = qx - fx0, fy = qy - fy0, fz = qz - fz0;
-    const int i = A.base + ((int)fz0 * v.rows + (int)fy0) * v.pitch + (int)fx0;
-    const int w = i >> 1;
-    const int hp = v.pitch >> 1, hs = (v.rows * v.pitch) >> 1;  // a row and a slab in words
-    const T* p = (i & 1) ? slot1 : slot;
-    const float2 c00 = ld_pair<T>(p, w), c10 = ld_pair<T>(p, w + hp);
-    const float2 c01 = ld_pair<T>(p, w + hs), c11 = ld_pair<T>(p, w + hs + hp);
+    float fx, fy, fz;
+    const int i = near_offset<T, BR>(v, A, qx, qy, qz, fx, fy, fz);
+    const int hp = SlotGeom<T, BR>::pitch(v) >> 1, hs = SlotGeom<T, BR>::slab(v) >> 1;  // a row and a slab in words
+    const T* p = ((i & 1) ? slot1 : slot) + (i & ~1);
+    const float2 c00 = ld_pair<T>(p, 0), c10 = ld_pair<T>(p, hp);
+    const float2 c01 = ld_pair<T>(p, hs), c11 = ld_pair<T>(p, hs + hp);
     const float a0 = fmaf(fx, c00.y - c00.x, c00.x), a1 = fmaf(fx, c10.y - c10.x, c10.x);
     const float a2 = fmaf(fx, c01.y - c01.x, c01.x), a3 = fmaf(fx, c11.y - c11.x, c11.x);
     const float b0 = fmaf(fy, a1 - a0, a0), b1 = fmaf(fy, a3 - a2, a2);
@@ -402,7 +416,10 @@ __device__ __forceinline__ int tf_node(int n, float vmin, float inv_range, float
 // Survey frame (1920 x 1080): sort-last 5.24 -> 4.59 ms, layered 0.506 -> 0.490,
 // marcher 0.473 -> 0.464; channel pairs (value, rise) as 8-byte loads: marcher 0.474,
 // layered 0.544.  The operations are those of the lookup below.
-template <int S>
+//
+// With RISE the second value of an interval is its rise, computed once here (entries
+// S 4 on) instead of by four subtractions a sample.
+template <int S, bool RISE = false>
 __device__ __forceinline__ void fill_table(float* __restrict__ tab, const TFDev& tf) {
     for (int i = threadIdx.x; i < tf.n; i += blockDim.x) {
         const float4 a = tf.tab[i];
@@ -410,10 +427,17 @@ __device__ __forceinline__ void fill_table(float* __restrict__ tab, const TFDev&
         tab[S + i] = a.y;
         tab[2 * S + i] = a.z;
         tab[3 * S + i] = a.w;
+        if (RISE) {
+            const float4 b = tf.tab[min(i + 1, tf.n - 1)];
+            tab[4 * S + i] = b.x - a.x;
+            tab[5 * S + i] = b.y - a.y;
+            tab[6 * S + i] = b.z - a.z;
+            tab[7 * S + i] = b.w - a.w;
+        }
     }
 }
 
-template <int S>
+template <int S, bool RISE = false>
 __device__ __forceinline__ float4 tf_lookup(const float* __restrict__ tab, int n, float vmin, float inv_range,
                                             float val) {
     float x;
@@ -421,6 +445,9 @@ __device__ __forceinline__ float4 tf_lookup(const float* __restrict__ tab, int n
     const float w = x - (float)i;
     const float* t = tab + i;
     const float4 a = make_float4(t[0], t[S], t[2 * S], t[3 * S]);
+    if (RISE)
+        return make_float4(fmaf(w, t[4 * S], a.x), fmaf(w, t[5 * S], a.y), fmaf(w, t[6 * S], a.z),
+                           fmaf(w, t[7 * S], a.w));
     const float4 b = make_float4(t[1], t[S + 1], t[2 * S + 1], t[3 * S + 1]);
     return make_float4(fmaf(w, b.x - a.x, a.x), fmaf(w, b.y - a.y, a.y),
                        fmaf(w, b.z - a.z, a.z), fmaf(w, b.w - a.w, a.w));

@@ -17,6 +17,7 @@ namespace vr {
 constexpr int kMaxLaunchCams = 32;   // cameras carried by value in one launch
 constexpr int kMaxTF = 1024;         // transfer-function entries
 constexpr int kTileW = 8, kTileH = 4; // pixels of one warp work item
+constexpr int kFastBrick = 128;      // the default brick edge, compiled into the marchers
 
 // One camera as the host keeps it (double precision; Sec. 3's off-axis
 // sub-windows are just other (l, t, du, dv)); kernels get it as a CamFF.
@@ -197,7 +198,7 @@ cudaError_t launch_repack(const float* src, long long src_z0, int bz0, int nlaye
                           void* pool, void* pool1, unsigned int* minmax, cudaStream_t s);
 // The marcher reads x-neighbour pairs with one load when p.vol.pool1 is set.
 cudaError_t launch_march(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s);
-int march_blocks_per_sm(vr_dtype dt, int mode, bool paired, int block);
+int march_blocks_per_sm(const MarchParams& p, vr_dtype dt, int block);
 // Layered composite of a cube in core: as launch_march, the samples owned and
 // positioned brick by brick as in launch_brick_partial.
 cudaError_t launch_march_layered(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s);
