@@ -765,9 +765,7 @@ vr_status render_ray(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
     P.ert = (float)ctx->opt.ert;
     P.samples = ctx->sample_counter;
     const int block = ctx->tune.block;
-    const bool paired = P.vol.pool1 != nullptr;
-    const int per_sm = layered ? layered_blocks_per_sm(ctx->dtype, paired, block)
-                               : march_blocks_per_sm(P, ctx->dtype, block);
+    const int per_sm = layered ? layered_blocks_per_sm(P, ctx->dtype, block) : march_blocks_per_sm(P, ctx->dtype, block);
     const int grid = ctx->num_sms * per_sm * block / 32;
     const long long img = (long long)P.width * P.height;
     if (ctx->ev_start) VR_CK(cudaEventRecord(ctx->ev_start, s), "vr_render: profiling event");

@@ -202,7 +202,7 @@ int march_blocks_per_sm(const MarchParams& p, vr_dtype dt, int block);
 // Layered composite of a cube in core: as launch_march, the samples owned and
 // positioned brick by brick as in launch_brick_partial.
 cudaError_t launch_march_layered(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s);
-int layered_blocks_per_sm(vr_dtype dt, bool paired, int block);
+int layered_blocks_per_sm(const MarchParams& p, vr_dtype dt, int block);
 cudaError_t launch_pixel_setup(const SetupParams& p, cudaStream_t s);
 cudaError_t launch_mip_finalize(const FinalizeParams& p, cudaStream_t s);
 // `cells` is per-context scratch of brick_cells_bytes(units) bytes (a counter and the

@@ -378,17 +378,60 @@ k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer
 // active (27 launches on the survey cube), set a ray up again in every brick,
 // carried its state through memory, and needed the bricks' order on the host;
 // here a pixel's set-up is done once and U samples' fetches are in flight at a time.
-// Survey frame (1024 x 1024 x 2048, 1920 x 1080, BF16): 3.27 -> 0.51 ms.  With paired
-// loads U = 4, 5, 6, 8 took 0.538, 0.515, 0.507, 0.538 ms.
+// Survey frame (1024 x 1024 x 2048, 1920 x 1080, BF16): 3.29 -> 0.46 ms, 0.47 of it before
+// the compiled geometry, rises and branch-free termination of k_march.  With paired
+// loads U = 4, 5, 6 take 0.475, 0.456, 0.464 ms.
 constexpr int kLayeredUnroll = 4;
-constexpr int kLayeredUnrollPaired = 6;
+constexpr int kLayeredUnrollPaired = 5;
+constexpr int kLayeredTF = 256;  // FAST: the default brick edge and tables up to this size, as in k_march
 
-template <typename T, bool PAIRED>
+// One brick's samples [0, n) at slot coordinates g + j e, composited onto (C, Tr); true
+// once 1 - Tr reaches ert.  CLAMP keeps the coordinates inside the slot.
+template <typename T, bool PAIRED, bool FAST, bool CLAMP>
+__device__ __forceinline__ bool layered_walk(const T* slot, const T* slot1, const VolDev& v, const TFDev& tf,
+                                             const float* s_tf, float3 g, float3 e, int n, float ert, float& C0,
+                                             float& C1, float& C2, float& Tr) {
+    constexpr int U = PAIRED ? kLayeredUnrollPaired : kLayeredUnroll;
+    constexpr int BR = FAST ? kFastBrick : 0, S = FAST ? kLayeredTF : kMaxTF;
+    const Anchor A{0.f, 0.f, 0.f, 0};  // offsets from the slot's first voxel
+    const float hi = (float)v.B + 0.999f;
+    bool done = false;
+    for (int i = 0; i < n && !done; i += U) {
+        float val[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const float fj = (float)min(i + q, n - 1);
+            float x = fmaf(fj, e.x, g.x), y = fmaf(fj, e.y, g.y), z = fmaf(fj, e.z, g.z);
+            if (CLAMP) {
+                x = fminf(fmaxf(x, 0.f), hi);
+                y = fminf(fmaxf(y, 0.f), hi);
+                z = fminf(fmaxf(z, 0.f), hi);
+            }
+            if constexpr (PAIRED) val[q] = fetch_near_pair<T, BR>(slot, slot1, v, A, x, y, z);
+            else val[q] = fetch_near<T, BR>(slot, v, A, x, y, z);
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const bool on = i + q < n && !done;  // else opacity 0: nothing changes
+            const float4 t = tf_lookup<S, FAST>(s_tf, tf.n, tf.vmin, tf.inv_range, val[q]);
+            const float a = on ? t.w : 0.f;
+            const float w = Tr * a;
+            C0 = fmaf(w, t.x, C0);
+            C1 = fmaf(w, t.y, C1);
+            C2 = fmaf(w, t.z, C2);
+            Tr = Tr * (1.f - a);
+            done = done || (on && 1.f - Tr >= ert);
+        }
+    }
+    return done;
+}
+
+template <typename T, bool PAIRED, bool FAST>
 __global__ void __launch_bounds__(256, 2)
 k_march_layered(const __grid_constant__ MarchParams P) {
-    constexpr int U = PAIRED ? kLayeredUnrollPaired : kLayeredUnroll;
-    __shared__ float s_tf[4 * kMaxTF];
-    fill_table<kMaxTF>(s_tf, P.tf);
+    constexpr int S = FAST ? kLayeredTF : kMaxTF;
+    __shared__ float s_tf[(FAST ? 8 : 4) * S];
+    fill_table<S, FAST>(s_tf, P.tf);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int tiles_per_cam = P.tiles_x * P.tiles_y;
@@ -457,33 +500,19 @@ k_march_layered(const __grid_constant__ MarchParams P) {
                     const T* slot = pool + base;
                     const T* slot1 = PAIRED ? pool1 + base : nullptr;
                     const ff fk = ff_of_int(k);
-                    const float gx = slot_coord(O[0], E[0], fk, b[0], B), gy = slot_coord(O[1], E[1], fk, b[1], B),
-                                gz = slot_coord(O[2], E[2], fk, b[2], B);
+                    const float3 g = make_float3(slot_coord(O[0], E[0], fk, b[0], B), slot_coord(O[1], E[1], fk, b[1], B),
+                                                 slot_coord(O[2], E[2], fk, b[2], B));
+                    const float3 e32 = make_float3(E[0].hi, E[1].hi, E[2].hi);
                     const int n = kb - k;
-                    for (int i = 0; i < n && !done; i += U) {
-                        float v[U];
-#pragma unroll
-                        for (int q = 0; q < U; ++q) {
-                            const float fj = (float)min(i + q, n - 1);
-                            const float x = fmaf(fj, E[0].hi, gx), y = fmaf(fj, E[1].hi, gy), z = fmaf(fj, E[2].hi, gz);
-                            if constexpr (PAIRED) v[q] = fetch_trilinear_pair<T>(slot, slot1, P.vol, x, y, z);
-                            else v[q] = fetch_trilinear<T>(slot, P.vol, x, y, z);
-                        }
-#pragma unroll
-                        for (int q = 0; q < U; ++q) {
-                            if (i + q >= n) break;
-                            const float4 t = tf_lookup<kMaxTF>(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v[q]);
-                            const float w = Tr * t.w;
-                            C0 = fmaf(w, t.x, C0);
-                            C1 = fmaf(w, t.y, C1);
-                            C2 = fmaf(w, t.z, C2);
-                            Tr = Tr * (1.f - t.w);
-                            if (1.f - Tr >= ert) {
-                                done = true;
-                                break;
-                            }
-                        }
-                    }
+                    // samples lie between the first and the last one: if both are inside the slot, all are
+                    const float fl = (float)(n - 1), hi = (float)B + 0.999f;
+                    const float x1 = fmaf(fl, e32.x, g.x), y1 = fmaf(fl, e32.y, g.y), z1 = fmaf(fl, e32.z, g.z);
+                    const bool inside = fminf(fminf(fminf(g.x, x1), fminf(g.y, y1)), fminf(g.z, z1)) >= 0.f &&
+                                        fmaxf(fmaxf(fmaxf(g.x, x1), fmaxf(g.y, y1)), fmaxf(g.z, z1)) <= hi;
+                    done = inside ? layered_walk<T, PAIRED, FAST, false>(slot, slot1, P.vol, P.tf, s_tf, g, e32, n, ert,
+                                                                         C0, C1, C2, Tr)
+                                  : layered_walk<T, PAIRED, FAST, true>(slot, slot1, P.vol, P.tf, s_tf, g, e32, n, ert,
+                                                                        C0, C1, C2, Tr);
                 }
                 k = kb;
 #pragma unroll
@@ -617,25 +646,33 @@ cudaError_t launch_brick_partial(const SortParams& p, vr_dtype dt, bool carried,
 }
 
 namespace {
-void* layered_ptr(vr_dtype dt, bool paired) {
-    if (dt == VR_F32) return reinterpret_cast<void*>(&k_march_layered<float, false>);
-    if (dt == VR_F16)
-        return paired ? reinterpret_cast<void*>(&k_march_layered<__half, true>)
-                      : reinterpret_cast<void*>(&k_march_layered<__half, false>);
-    return paired ? reinterpret_cast<void*>(&k_march_layered<__nv_bfloat16, true>)
-                  : reinterpret_cast<void*>(&k_march_layered<__nv_bfloat16, false>);
+template <typename T>
+void* layered_t(bool paired, bool fast) {
+    if constexpr (sizeof(T) == 2) {
+        if (paired)
+            return fast ? reinterpret_cast<void*>(&k_march_layered<T, true, true>)
+                        : reinterpret_cast<void*>(&k_march_layered<T, true, false>);
+    }
+    return fast ? reinterpret_cast<void*>(&k_march_layered<T, false, true>)
+                : reinterpret_cast<void*>(&k_march_layered<T, false, false>);
+}
+
+void* layered_ptr(vr_dtype dt, const MarchParams& p) {
+    const bool paired = p.vol.pool1 != nullptr, fast = p.vol.B == kFastBrick && p.tf.n <= kLayeredTF;
+    if (dt == VR_F32) return layered_t<float>(paired, fast);
+    return dt == VR_F16 ? layered_t<__half>(paired, fast) : layered_t<__nv_bfloat16>(paired, fast);
 }
 }  // namespace
 
-int layered_blocks_per_sm(vr_dtype dt, bool paired, int block) {
+int layered_blocks_per_sm(const MarchParams& p, vr_dtype dt, int block) {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, layered_ptr(dt, paired), block, 0) != cudaSuccess) return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, layered_ptr(dt, p), block, 0) != cudaSuccess) return 1;
     return n > 0 ? n : 1;
 }
 
 cudaError_t launch_march_layered(const MarchParams& p, vr_dtype dt, int grid, int block, cudaStream_t s) {
     void* args[] = {const_cast<MarchParams*>(&p)};
-    return cudaLaunchKernel(layered_ptr(dt, p.vol.pool1 != nullptr), dim3(grid), dim3(block), args, 0, s);
+    return cudaLaunchKernel(layered_ptr(dt, p), dim3(grid), dim3(block), args, 0, s);
 }
 
 cudaError_t launch_sortlast_fold(const SortParams& p, cudaStream_t s) {
