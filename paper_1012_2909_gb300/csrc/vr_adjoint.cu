@@ -30,8 +30,13 @@ constexpr int kAdjThreads = 128;
 constexpr int kAdjWarps = kAdjThreads / 32;
 constexpr int kAdjMaxChunks = 320;  // 32-sample transmittance checkpoints per ray
 constexpr int kAdjFlush = 8;        // chunks collected in the table histograms at a time
-constexpr int kAdjKeep = 4;         // chunks whose samples the forward pass keeps for the reverse pass
+constexpr int kAdjKeep = 6;         // chunks whose samples the forward pass keeps for the reverse pass
 constexpr int kDevTooManySegments = 2;
+
+// Tables of up to kAdjTF entries and the default brick edge are compiled in (FAST): the
+// table's arrays are S entries apart, S = 0 standing for its length.
+constexpr int kAdjTF = 256;
+template <int S> __device__ __forceinline__ int stride(int n) { return S ? S : n; }
 
 struct TFGrad {
     int i;
@@ -39,6 +44,7 @@ struct TFGrad {
     float4 rgba, slope;
 };
 
+template <int S>
 __device__ __forceinline__ TFGrad tf_eval(const float* __restrict__ tab, int n, float vmin,
                                           float inv_range, float val) {
     TFGrad r;
@@ -48,23 +54,26 @@ __device__ __forceinline__ TFGrad tf_eval(const float* __restrict__ tab, int n, 
     const float x = u * (float)(n - 1);
     r.i = min((int)x, n - 2);
     r.w = x - (float)r.i;
+    const int d = stride<S>(n);
     const float* t = tab + r.i;
-    const float4 a = make_float4(t[0], t[n], t[2 * n], t[3 * n]);
-    const float4 b = make_float4(t[1], t[n + 1], t[2 * n + 1], t[3 * n + 1]);
-    r.rgba = make_float4(fmaf(r.w, b.x - a.x, a.x), fmaf(r.w, b.y - a.y, a.y), fmaf(r.w, b.z - a.z, a.z),
-                         fmaf(r.w, b.w - a.w, a.w));
+    const float4 a = make_float4(t[0], t[d], t[2 * d], t[3 * d]);
+    const float4 b = make_float4(t[1], t[d + 1], t[2 * d + 1], t[3 * d + 1]);
+    const float4 up = make_float4(b.x - a.x, b.y - a.y, b.z - a.z, b.w - a.w);
+    r.rgba = make_float4(fmaf(r.w, up.x, a.x), fmaf(r.w, up.y, a.y), fmaf(r.w, up.z, a.z), fmaf(r.w, up.w, a.w));
     const float s = inside ? (float)(n - 1) * inv_range : 0.f;
-    r.slope = make_float4((b.x - a.x) * s, (b.y - a.y) * s, (b.z - a.z) * s, (b.w - a.w) * s);
+    r.slope = make_float4(up.x * s, up.y * s, up.z * s, up.w * s);
     return r;
 }
 
 // Opacity alone, of the table above.
+template <int S>
 __device__ __forceinline__ float tf_alpha(const float* __restrict__ tab, int n, float vmin, float inv_range,
                                           float val) {
     float x;
     const int i = tf_node(n, vmin, inv_range, val, x);
     const float w = x - (float)i;
-    const float a = tab[3 * n + i], b = tab[3 * n + i + 1];
+    const float* t = tab + 3 * stride<S>(n) + i;
+    const float a = t[0], b = t[1];
     return fmaf(w, b - a, a);
 }
 
@@ -76,32 +85,41 @@ __device__ __forceinline__ void scatter_voxels(float* __restrict__ dvol, const V
     const float fx = gx - fx0, fy = gy - fy0, fz = gz - fz0;
     // slot index s <-> cube index b*B + s - 1, clamped to the cube like the ghost layer
     const int x0 = bx * v.B + (int)fx0 - 1, y0 = by * v.B + (int)fy0 - 1, z0 = bz * v.B + (int)fz0 - 1;
-    const int xs[2] = {min(max(x0, 0), v.nx - 1), min(max(x0 + 1, 0), v.nx - 1)};
-    const int ys[2] = {min(max(y0, 0), v.ny - 1), min(max(y0 + 1, 0), v.ny - 1)};
-    const int zs[2] = {min(max(z0, 0), v.nz - 1), min(max(z0 + 1, 0), v.nz - 1)};
-    const float wx[2] = {1.f - fx, fx}, wy[2] = {1.f - fy, fy}, wz[2] = {1.f - fz, fz};
+    const int xl = min(max(x0, 0), v.nx - 1), yl = min(max(y0, 0), v.ny - 1), zl = min(max(z0, 0), v.nz - 1);
+    const int dx = min(max(x0 + 1, 0), v.nx - 1) - xl;  // 0 where both clamp to the same voxel, else 1
+    const long long dy = min(max(y0 + 1, 0), v.ny - 1) > yl ? v.nx : 0;
+    const long long dz = min(max(z0 + 1, 0), v.nz - 1) > zl ? (long long)v.nx * v.ny : 0;
+    float* p = dvol + ((long long)zl * v.ny + yl) * v.nx + xl;
+    const float wz[2] = {(1.f - fz) * dv, fz * dv};
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-        const float w = wx[dx] * wy[dy] * wz[dz];
-        const long long idx = ((long long)zs[dz] * v.ny + ys[dy]) * v.nx + xs[dx];
-        atomicAdd(dvol + idx, w * dv);
+    for (int c = 0; c < 4; ++c) {
+        float* q = p + (c & 1 ? dy : 0) + (c >> 1 ? dz : 0);
+        const float w = wz[c >> 1] * (c & 1 ? fy : 1.f - fy);
+        if (dx && (reinterpret_cast<uintptr_t>(q) & 7) == 0) {  // an aligned x-pair in one reduction
+            asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(q), "f"(w * (1.f - fx)), "f"(w * fx)
+                         : "memory");
+        } else {
+            atomicAdd(q, w * (1.f - fx));
+            atomicAdd(q + dx, w * fx);
+        }
     }
 }
 
-// g: the block's table gradient, channel-major (g[c * n + i]), so that the lanes
+// g: the block's table gradient, channel-major (g[c * stride + i]), so that the lanes
 // of one atomic instruction fall on banks by table entry, not by entry mod 8.
+template <int S>
 __device__ __forceinline__ void add_tf(float* __restrict__ g, int n, const TFGrad& t, float4 gc) {
     const float w1 = t.w, w0 = 1.f - t.w;
+    const int d = stride<S>(n);
     float* a = g + t.i;
     atomicAdd(a, w0 * gc.x);
-    atomicAdd(a + n, w0 * gc.y);
-    atomicAdd(a + 2 * n, w0 * gc.z);
-    atomicAdd(a + 3 * n, w0 * gc.w);
+    atomicAdd(a + d, w0 * gc.y);
+    atomicAdd(a + 2 * d, w0 * gc.z);
+    atomicAdd(a + 3 * d, w0 * gc.w);
     atomicAdd(a + 1, w1 * gc.x);
-    atomicAdd(a + n + 1, w1 * gc.y);
-    atomicAdd(a + 2 * n + 1, w1 * gc.z);
-    atomicAdd(a + 3 * n + 1, w1 * gc.w);
+    atomicAdd(a + d + 1, w1 * gc.y);
+    atomicAdd(a + 2 * d + 1, w1 * gc.z);
+    atomicAdd(a + 3 * d + 1, w1 * gc.w);
 }
 
 // One warp per ray, its lanes on 32 consecutive samples (a chunk).  A warp
@@ -117,7 +135,7 @@ __device__ __forceinline__ void add_tf(float* __restrict__ g, int n, const TFGra
 // maximal sample.  Sample positions: the float-float ray from the set-up, one
 // float-float anchor per chunk, lane offsets in FP32, each lane
 // reading the brick that holds its sample (the ghost layer makes any brick
-// within half a voxel give the same value).
+// within half a voxel give the same value, and keeps the corners inside the slot).
 //
 // Table gradient.  A float atomicAdd in shared memory is a compare-and-swap loop,
 // repeated while lanes meet on an entry; eight a sample (4 channels x 2 entries) took
@@ -127,18 +145,21 @@ __device__ __forceinline__ void add_tf(float* __restrict__ g, int n, const TFGra
 // the entries it touched:
 //   colour: dL/dc_k = dL/dC T_k a_k, one weight T_k a_k for all three channels; the
 //     weights of a ray add up to at most 1 and are kept in units of 2^-30;
-//   alpha: |dL/da_k| <= S = |g.w| + 2 cmax (|g.x| + |g.y| + |g.z|), cmax the table's
-//     largest colour; scaled by 2^-E, 2^E <= S < 2^(E+1), and kept in units of n / 2^29, n
+//   alpha: |dL/da_k| <= M = |g.w| + 2 cmax (|g.x| + |g.y| + |g.z|), cmax the table's
+//     largest colour; scaled by 2^-E, 2^E <= M < 2^(E+1), and kept in units of n / 2^29, n
 //     the samples collected together (at most 256 of a ray), so that no sum leaves 31
 //     bits.
-// A sample is rounded by 2^-22 S at most, less than the FP32 sums over the rays round.
-// This needs opacities in [0, 1] and a finite S; other tables, and rays whose dL/dI is
+// A sample is rounded by 2^-22 M at most, less than the FP32 sums over the rays round.
+// This needs opacities in [0, 1] and a finite M; other tables, and rays whose dL/dI is
 // not finite, take the FP32 atomics.
 //
-// Bound by L1 data wavefronts (gathers, scans, the voxel atomics).  Six CTAs an SM (85
-// registers).  16 views of 512 x 512 on 256^3 FP32, forward and backward: 11.7 -> 7.9 ms
-// (k_adjoint 10.4 -> 6.5 ms).  kAdjKeep = 2, 4, 6 at five CTAs: 8.79, 8.47, 8.40 ms; six
-// CTAs with 4, 6: 8.31, 8.37 ms; seven CTAs spill: 8.83 ms.
+// Bound by L1 data wavefronts and the voxel atomics in L2 (both 78 % busy), with issue
+// slots at 63 %: two passes over a chunk took some 1100 warp instructions before the
+// anchors of a ray's chunks were made together, the default brick edge and table stride
+// compiled in, the voxel addresses taken from one base and aligned x-pairs reduced
+// together.  16 views of 512 x 512 on 256^3 FP32, forward and backward: 11.6 -> 7.2 ms (8.0
+// before these).  Five CTAs an SM and kAdjKeep = 6: 7.73 ms; six CTAs and 4: 7.79; five and
+// 4: 7.81 (one seed).
 struct RaySetup {
     float o_hi[3], o_lo[3], e_hi[3], e_lo[3];
     int k0, k1;
@@ -165,59 +186,80 @@ __device__ __forceinline__ int anchor_axis(ff p, const VolDev& v, int nb, float&
     return b;
 }
 
-__device__ __forceinline__ void lane_sample(const RaySetup& r, int k, int lane, float3 e32, const VolDev& v,
-                                            LaneSample& s) {
-    const ff fk = ff_of_int(k);  // exact for any sample index
+// Brick index and slot coordinate of one sample.
+struct __align__(16) SampleAnchor {
     float gx, gy, gz;
-    const int bx0 = anchor_axis(ff_add(ff{r.o_hi[0], r.o_lo[0]}, ff_mul(ff{r.e_hi[0], r.e_lo[0]}, fk)), v, v.nbx, gx);
-    const int by0 = anchor_axis(ff_add(ff{r.o_hi[1], r.o_lo[1]}, ff_mul(ff{r.e_hi[1], r.e_lo[1]}, fk)), v, v.nby, gy);
-    const int bz0 = anchor_axis(ff_add(ff{r.o_hi[2], r.o_lo[2]}, ff_mul(ff{r.e_hi[2], r.e_lo[2]}, fk)), v, v.nbz, gz);
+    int bx, by, bz;
+};
+
+__device__ __forceinline__ void sample_anchor(const RaySetup& r, int k, const VolDev& v, SampleAnchor& A) {
+    const ff fk = ff_of_int(k);  // exact for any sample index
+    A.bx = anchor_axis(ff_add(ff{r.o_hi[0], r.o_lo[0]}, ff_mul(ff{r.e_hi[0], r.e_lo[0]}, fk)), v, v.nbx, A.gx);
+    A.by = anchor_axis(ff_add(ff{r.o_hi[1], r.o_lo[1]}, ff_mul(ff{r.e_hi[1], r.e_lo[1]}, fk)), v, v.nby, A.gy);
+    A.bz = anchor_axis(ff_add(ff{r.o_hi[2], r.o_lo[2]}, ff_mul(ff{r.e_hi[2], r.e_lo[2]}, fk)), v, v.nbz, A.gz);
+}
+
+// This lane's sample of chunk c.  The float-float anchors of 32 chunks are made at once, a
+// chunk a lane, and kept in shared memory (anchors: the 32 of chunks 32 group ..), instead
+// of by every lane for every chunk in both passes.  All lanes take part; those past the
+// ray's end get a sample outside the cube, to be ignored.
+__device__ __forceinline__ LaneSample lane_sample(const RaySetup& r, int c, int lane, float3 e32, const VolDev& v,
+                                                  SampleAnchor* anchors, int& group) {
+    if (c >> 5 != group) {
+        group = c >> 5;
+        __syncwarp();
+        sample_anchor(r, r.k0 + 32 * (32 * group + lane), v, anchors[lane]);
+        __syncwarp();
+    }
+    const SampleAnchor A = anchors[c & 31];
     const float fl = (float)lane;
-    gx = fmaf(fl, e32.x, gx);
-    gy = fmaf(fl, e32.y, gy);
-    gz = fmaf(fl, e32.z, gz);
-    const float B = (float)v.B, invB = 1.0f / B;
-    const int bx = min(max(bx0 + (int)floorf((gx - 0.5f) * invB), 0), v.nbx - 1);
-    const int by = min(max(by0 + (int)floorf((gy - 0.5f) * invB), 0), v.nby - 1);
-    const int bz = min(max(bz0 + (int)floorf((gz - 0.5f) * invB), 0), v.nbz - 1);
-    s.gx = gx - (float)((bx - bx0) << v.log2B);
-    s.gy = gy - (float)((by - by0) << v.log2B);
-    s.gz = gz - (float)((bz - bz0) << v.log2B);
-    s.bx = bx;
-    s.by = by;
-    s.bz = bz;
-    s.base = (long long)v.table[(bz * v.nby + by) * v.nbx + bx] * v.slot_elems;
+    const float gx = fmaf(fl, e32.x, A.gx), gy = fmaf(fl, e32.y, A.gy), gz = fmaf(fl, e32.z, A.gz);
+    const float invB = 1.0f / (float)v.B;
+    LaneSample s;
+    s.bx = min(max(A.bx + (int)floorf((gx - 0.5f) * invB), 0), v.nbx - 1);
+    s.by = min(max(A.by + (int)floorf((gy - 0.5f) * invB), 0), v.nby - 1);
+    s.bz = min(max(A.bz + (int)floorf((gz - 0.5f) * invB), 0), v.nbz - 1);
+    s.gx = gx - (float)((s.bx - A.bx) << v.log2B);
+    s.gy = gy - (float)((s.by - A.by) << v.log2B);
+    s.gz = gz - (float)((s.bz - A.bz) << v.log2B);
+    // a cube in core: brick b is slot b
+    s.base = (long long)((s.bz * v.nby + s.by) * v.nbx + s.bx) * v.slot_elems;
+    return s;
 }
 
 constexpr float kColourUnits = 1073741824.f;  // 2^30
 constexpr float kAlphaUnits = 536870912.f;    // 2^29
 
-template <typename T, int MODE>
-__global__ void __launch_bounds__(kAdjThreads, 6)
+template <typename T, int MODE, bool FAST>
+__global__ void __launch_bounds__(kAdjThreads, 5)
 k_adjoint(const __grid_constant__ AdjParams P) {
     constexpr unsigned int FULL = 0xffffffffu;
     // dynamic, by the size of the table: the table and the block's gradient of it, both
     // channel-major, then a pair of histograms per warp
     extern __shared__ __align__(16) float s_dyn[];
-    const int ntf = P.tf.n;
+    constexpr int S = FAST ? kAdjTF : 0, BR = FAST ? kFastBrick : 0;
+    const int ntf = P.tf.n, sd = stride<S>(ntf);
+    const Anchor slot0{0.f, 0.f, 0.f, 0};  // fetches from the slot's first voxel
     float* s_tf = s_dyn;
-    float* g_tf = s_dyn + 4 * ntf;
+    float* g_tf = s_dyn + 4 * sd;
     __shared__ RaySetup s_ray[kAdjWarps][32];
+    __shared__ SampleAnchor s_anchor[kAdjWarps][32];
     __shared__ float2 s_keep[kAdjWarps][MODE == VR_COMPOSITE ? kAdjKeep * 32 : 1];
     for (int i = threadIdx.x; i < ntf; i += blockDim.x) {
         const float4 t = P.tf.tab[i];
         s_tf[i] = t.x;
-        s_tf[ntf + i] = t.y;
-        s_tf[2 * ntf + i] = t.z;
-        s_tf[3 * ntf + i] = t.w;
+        s_tf[sd + i] = t.y;
+        s_tf[2 * sd + i] = t.z;
+        s_tf[3 * sd + i] = t.w;
     }
-    for (int i = threadIdx.x; i < (4 + (MODE == VR_COMPOSITE ? 2 * kAdjWarps : 0)) * ntf; i += blockDim.x)
+    for (int i = threadIdx.x; i < (4 + (MODE == VR_COMPOSITE ? 2 * kAdjWarps : 0)) * sd; i += blockDim.x)
         g_tf[i] = 0.f;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int* hist_c = reinterpret_cast<int*>(g_tf + 4 * ntf) + warp * 2 * ntf;
-    int* hist_a = hist_c + ntf;
+    int* hist_c = reinterpret_cast<int*>(g_tf + 4 * sd) + warp * 2 * sd;
+    int* hist_a = hist_c + sd;
     float2* keep = s_keep[warp];
+    SampleAnchor* anchors = s_anchor[warp];
     const int tiles_per_cam = P.tiles_x * P.tiles_y;
     const int total = tiles_per_cam * P.ncams;
     const T* __restrict__ pool = static_cast<const T*>(P.vol.pool);
@@ -264,6 +306,7 @@ k_adjoint(const __grid_constant__ AdjParams P) {
             const RaySetup r = s_ray[warp][who];
             const float3 e32 = make_float3(r.e_hi[0], r.e_hi[1], r.e_hi[2]);
             const float4 gI = r.g;
+            int group = -1;
 
             if (MODE == VR_MIP) {
                 unsigned int best = ord_enc_f(-INFINITY);
@@ -272,10 +315,9 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                 for (int k = r.k0; k < r.k1; k += 32) {
                     const bool act = k + lane < r.k1;
                     float v = -INFINITY;
+                    const LaneSample ls = lane_sample(r, (k - r.k0) >> 5, lane, e32, P.vol, anchors, group);
                     if (act) {
-                        LaneSample ls;
-                        lane_sample(r, k, lane, e32, P.vol, ls);
-                        v = fetch_trilinear<T>(pool + ls.base, P.vol, ls.gx, ls.gy, ls.gz);
+                        v = fetch_near<T, BR>(pool + ls.base, P.vol, slot0, ls.gx, ls.gy, ls.gz);
                     }
                     const unsigned int e = act ? ord_enc_f(v) : 0u;
                     const unsigned int cmax = __reduce_max_sync(FULL, e);
@@ -288,11 +330,11 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                 }
                 if (kmax < 0) continue;
                 if (lane == 0) {
-                    const TFGrad t = tf_eval(s_tf, ntf, P.tf.vmin, P.tf.inv_range, m);
-                    add_tf(g_tf, ntf, t, gI);
+                    const TFGrad t = tf_eval<S>(s_tf, ntf, P.tf.vmin, P.tf.inv_range, m);
+                    add_tf<S>(g_tf, ntf, t, gI);
                     if (P.dvol) {
-                        LaneSample ls;
-                        lane_sample(r, kmax, 0, e32, P.vol, ls);
+                        SampleAnchor ls;
+                        sample_anchor(r, kmax, P.vol, ls);
                         const float dv = gI.x * t.slope.x + gI.y * t.slope.y + gI.z * t.slope.z + gI.w * t.slope.w;
                         scatter_voxels(P.dvol, P.vol, ls.bx, ls.by, ls.bz, ls.gx, ls.gy, ls.gz, dv);
                     }
@@ -318,11 +360,10 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                     const int n = min(32, r.k1 - k);
                     const bool act = lane < n;
                     float q = 1.f, v = 0.f;
+                    const LaneSample ls = lane_sample(r, nch, lane, e32, P.vol, anchors, group);
                     if (act) {
-                        LaneSample ls;
-                        lane_sample(r, k, lane, e32, P.vol, ls);
-                        v = fetch_trilinear<T>(pool + ls.base, P.vol, ls.gx, ls.gy, ls.gz);
-                        q = 1.f - tf_alpha(s_tf, ntf, P.tf.vmin, P.tf.inv_range, v);
+                        v = fetch_near<T, BR>(pool + ls.base, P.vol, slot0, ls.gx, ls.gy, ls.gz);
+                        q = 1.f - tf_alpha<S>(s_tf, ntf, P.tf.vmin, P.tf.inv_range, v);
                     }
                     float incl = q;
 #pragma unroll
@@ -348,33 +389,32 @@ k_adjoint(const __grid_constant__ AdjParams P) {
             }
             __syncwarp();
             // fixed-point units of this ray's alpha gradients (see above)
-            const float S = fabsf(gI.w) + 2.f * P.tf_cmax * (fabsf(gI.x) + fabsf(gI.y) + fabsf(gI.z));
-            const bool fixed = P.tf_unit && S < 1e30f;
-            const float p2 = pow2_recip(S);
+            const float bound = fabsf(gI.w) + 2.f * P.tf_cmax * (fabsf(gI.x) + fabsf(gI.y) + fabsf(gI.z));
+            const bool fixed = P.tf_unit && bound < 1e30f;
+            const float p2 = pow2_recip(bound);
             const float to_units = kAlphaUnits / (float)min(32 * (nch - 1) + n_last, 32 * kAdjFlush);
             const float from_units = 1.f / to_units / p2;
             int e_lo = ntf, e_hi = 0;  // entries touched by this lane's samples
             // ---- reverse: chunks back to front, suffix "over" scan within a chunk
             float Rc = 0.f, Pc = 1.f;
             for (int c = nch - 1; c >= 0; --c) {
-                const int k = r.k0 + 32 * c;
                 const int n = c == nch - 1 ? n_last : 32;
                 const bool act = lane < n;
                 const float ckT = __shfl_sync(FULL, c < 32 ? ck0 : ck[(c >> 5) - 1], c & 31);
                 TFGrad t;
                 LaneSample ls;
+                if (c >= kAdjKeep || P.dvol) ls = lane_sample(r, c, lane, e32, P.vol, anchors, group);
                 float a = 0.f, s = 0.f, incl = 1.f;
                 if (act) {
                     float v;
-                    if (c >= kAdjKeep || P.dvol) lane_sample(r, k, lane, e32, P.vol, ls);
                     if (c < kAdjKeep) {
                         const float2 kv = keep[c * 32 + lane];
                         v = kv.x;
                         incl = kv.y;
                     } else {
-                        v = fetch_trilinear<T>(pool + ls.base, P.vol, ls.gx, ls.gy, ls.gz);
+                        v = fetch_near<T, BR>(pool + ls.base, P.vol, slot0, ls.gx, ls.gy, ls.gz);
                     }
-                    t = tf_eval(s_tf, ntf, P.tf.vmin, P.tf.inv_range, v);
+                    t = tf_eval<S>(s_tf, ntf, P.tf.vmin, P.tf.inv_range, v);
                     a = t.rgba.w;
                     s = gI.x * t.rgba.x + gI.y * t.rgba.y + gI.z * t.rgba.z;
                 }
@@ -424,7 +464,7 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                         e_lo = min(e_lo, t.i);
                         e_hi = max(e_hi, t.i + 1);
                     } else {
-                        add_tf(g_tf, ntf, t, make_float4(gI.x * wk, gI.y * wk, gI.z * wk, ga));
+                        add_tf<S>(g_tf, ntf, t, make_float4(gI.x * wk, gI.y * wk, gI.z * wk, ga));
                     }
                     if (P.dvol) {
                         const float dv = wk * (gI.x * t.slope.x + gI.y * t.slope.y + gI.z * t.slope.z) + ga * t.slope.w;
@@ -442,9 +482,9 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                             hist_a[e] = 0;
                             const float h = (float)hc * (1.f / kColourUnits);
                             atomicAdd(g_tf + e, gI.x * h);
-                            atomicAdd(g_tf + ntf + e, gI.y * h);
-                            atomicAdd(g_tf + 2 * ntf + e, gI.z * h);
-                            atomicAdd(g_tf + 3 * ntf + e, (float)hg * from_units);
+                            atomicAdd(g_tf + sd + e, gI.y * h);
+                            atomicAdd(g_tf + 2 * sd + e, gI.z * h);
+                            atomicAdd(g_tf + 3 * sd + e, (float)hg * from_units);
                         }
                     }
                     e_lo = ntf;
@@ -459,7 +499,7 @@ k_adjoint(const __grid_constant__ AdjParams P) {
     __syncthreads();
     // block partial, entry-major (ntf x 4)
     float* out = P.tf_partials + (size_t)blockIdx.x * ntf * 4;
-    for (int i = threadIdx.x; i < ntf * 4; i += blockDim.x) out[i] = g_tf[(i & 3) * ntf + (i >> 2)];
+    for (int i = threadIdx.x; i < ntf * 4; i += blockDim.x) out[i] = g_tf[(i & 3) * sd + (i >> 2)];
 }
 
 // Final reduction of the per-block table partials, in FP64 (the only FP64
@@ -483,40 +523,39 @@ k_tfgrad_reduce(const float* __restrict__ partials, int nblocks, int nval, float
     }
 }
 
-template <typename T, int MODE>
-void* adj_ptr() {
-    return reinterpret_cast<void*>(&k_adjoint<T, MODE>);
+template <typename T>
+void* adj_t(int mode, bool fast) {
+    if (mode == VR_MIP)
+        return fast ? reinterpret_cast<void*>(&k_adjoint<T, VR_MIP, true>)
+                    : reinterpret_cast<void*>(&k_adjoint<T, VR_MIP, false>);
+    return fast ? reinterpret_cast<void*>(&k_adjoint<T, VR_COMPOSITE, true>)
+                : reinterpret_cast<void*>(&k_adjoint<T, VR_COMPOSITE, false>);
 }
 
-void* adj_pick(vr_dtype dt, int mode) {
-    if (dt == VR_F32) return mode == VR_MIP ? adj_ptr<float, VR_MIP>() : adj_ptr<float, VR_COMPOSITE>();
-    if (dt == VR_F16) return mode == VR_MIP ? adj_ptr<__half, VR_MIP>() : adj_ptr<__half, VR_COMPOSITE>();
-    return mode == VR_MIP ? adj_ptr<__nv_bfloat16, VR_MIP>() : adj_ptr<__nv_bfloat16, VR_COMPOSITE>();
+// The kernel for p and its dynamic shared memory: table, its gradient, two histograms a warp.
+void* adj_pick(const AdjParams& p, vr_dtype dt, size_t& smem) {
+    const bool fast = p.vol.B == kFastBrick && p.tf.n <= kAdjTF;
+    smem = (size_t)(fast ? kAdjTF : p.tf.n) * sizeof(float) * (8 + (p.mode == VR_COMPOSITE ? 2 * kAdjWarps : 0));
+    void* f = dt == VR_F32   ? adj_t<float>(p.mode, fast)
+              : dt == VR_F16 ? adj_t<__half>(p.mode, fast)
+                             : adj_t<__nv_bfloat16>(p.mode, fast);
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess ? f : nullptr;
 }
 
 }  // namespace
 
-int adjoint_threads() { return kAdjThreads; }
-
-// dynamic shared memory of k_adjoint: table, its gradient, two histograms a warp
-size_t adj_smem(int mode, int ntf) {
-    return (size_t)ntf * sizeof(float) * (8 + (mode == VR_COMPOSITE ? 2 * kAdjWarps : 0));
-}
-
-int adjoint_blocks_per_sm(vr_dtype dt, int mode, int ntf) {
-    const size_t smem = adj_smem(mode, ntf);
-    void* f = adj_pick(dt, mode);
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 1;
+int adjoint_blocks_per_sm(const AdjParams& p, vr_dtype dt) {
+    size_t smem;
+    void* f = adj_pick(p, dt, smem);
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, kAdjThreads, smem) != cudaSuccess) return 1;
+    if (!f || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, kAdjThreads, smem) != cudaSuccess) return 1;
     return n > 0 ? n : 1;
 }
 
 cudaError_t launch_adjoint(const AdjParams& p, vr_dtype dt, int grid, cudaStream_t s) {
-    const size_t smem = adj_smem(p.mode, p.tf.n);
-    void* f = adj_pick(dt, p.mode);
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    size_t smem;
+    void* f = adj_pick(p, dt, smem);
+    if (!f) return cudaGetLastError();
     void* args[] = {const_cast<AdjParams*>(&p)};
     return cudaLaunchKernel(f, dim3(grid), dim3(kAdjThreads), args, smem, s);
 }

@@ -1635,19 +1635,6 @@ vr_status vr_render_backward(vr_ctx* ctx, vr_mode mode, const float* dL_dimg, fl
     const int ncams = (int)ctx->cams.size();
     const int nbatch = (ncams + kMaxLaunchCams - 1) / kMaxLaunchCams;
     const int ntf = (int)ctx->tf.size();
-    const int grid = ctx->num_sms * adjoint_blocks_per_sm(ctx->dtype, mode, ntf);
-    const size_t need = (size_t)nbatch * grid * ntf * 4;
-    if (need > ctx->tf_partials_n) {
-        if (ctx->tf_partials) cudaFree(ctx->tf_partials);
-        ctx->tf_partials = nullptr;
-        ctx->tf_partials_n = 0;
-        VR_CK(cudaMalloc(&ctx->tf_partials, need * sizeof(float)), "vr_render_backward: partials");
-        ctx->tf_partials_n = need;
-    }
-    if (dL_dvol)
-        VR_CK(cudaMemsetAsync(dL_dvol, 0, sizeof(float) * (size_t)ctx->nx * ctx->ny * ctx->nz, s),
-              "vr_render_backward: clear dL_dvol");
-    VR_CK(cudaMemsetAsync(ctx->work, 0, sizeof(int) * nbatch, s), "vr_render_backward: scheduler reset");
     AdjParams P;
     std::memset(&P, 0, sizeof(P));
     P.vol = vol_dev(ctx);
@@ -1666,6 +1653,19 @@ vr_status vr_render_backward(vr_ctx* ctx, vr_mode mode, const float* dL_dimg, fl
     }
     P.dvol = dL_dvol;
     P.status = ctx->status_dev;
+    const int grid = ctx->num_sms * adjoint_blocks_per_sm(P, ctx->dtype);
+    const size_t need = (size_t)nbatch * grid * ntf * 4;
+    if (need > ctx->tf_partials_n) {
+        if (ctx->tf_partials) cudaFree(ctx->tf_partials);
+        ctx->tf_partials = nullptr;
+        ctx->tf_partials_n = 0;
+        VR_CK(cudaMalloc(&ctx->tf_partials, need * sizeof(float)), "vr_render_backward: partials");
+        ctx->tf_partials_n = need;
+    }
+    if (dL_dvol)
+        VR_CK(cudaMemsetAsync(dL_dvol, 0, sizeof(float) * (size_t)ctx->nx * ctx->ny * ctx->nz, s),
+              "vr_render_backward: clear dL_dvol");
+    VR_CK(cudaMemsetAsync(ctx->work, 0, sizeof(int) * nbatch, s), "vr_render_backward: scheduler reset");
     const long long img = (long long)P.width * P.height;
     for (int b = 0; b < nbatch; ++b) {
         const int c0 = b * kMaxLaunchCams;
