@@ -71,6 +71,7 @@ struct vr_ctx {
     bool has_tmap_part = false;
     vr_path path = VR_PATH_AUTO;
     vr_tuning tune{8, 4, 256, 8};  // tile_w, tile_h, block, group
+    bool group_set = false;        // the caller or the autotuner chose the group
     bool graph_mode = false;
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph_exec = nullptr;
@@ -823,6 +824,30 @@ FinalizeParams finalize_params(const vr_ctx* ctx) {
     return p;
 }
 
+// Lanes per ray segment of a staged-cell pass over views like `cd`: the tuning's where the
+// caller or the autotuner set one, else by the length of the segments and the spacing of
+// the rays at the cube's centre.  Fewer lanes waste less on a segment's last step, and pay
+// where neighbouring groups march segments of one length: in the short segments of FP32
+// cells (16 voxels thick: 1721 x 1721 x 1025 at 1.0 voxels a pixel 18.9 ms with 4 lanes and
+// 19.7 with 8; equal within 1 % up to 3 voxels a pixel), and with 16-bit cells where the
+// rays are at most a voxel apart (2048 x 2048 x 1024 on 25 panels: 0.66 voxels 49.4 and
+// 53.3 ms, 0.99 25.6 and 26.0; 1.31 16.6 and 16.3; 1024 x 1024 x 2048 at 2.7 voxels 2.57 and
+// 2.27).
+int pass_group(const vr_ctx* ctx, const CamDev& cd) {
+    if (ctx->group_set) return ctx->tune.group;
+    if (ctx->dtype == VR_F32) return 4;
+    const double c[3] = {0.5 * (double)ctx->nx, 0.5 * (double)ctx->ny, 0.5 * (double)ctx->nz};
+    auto len2 = [](const double* v) { return v[0] * v[0] + v[1] * v[1] + v[2] * v[2]; };
+    double scale = 1.0;  // of the window at the cube's centre
+    if (cd.type == 1) {
+        scale = 0.0;
+        for (int a = 0; a < 3; ++a) scale += (c[a] - cd.eye[a]) * cd.fwd[a];
+        scale = std::fabs(scale) / len2(cd.fwd);
+    }
+    const double area = std::fabs(cd.du * cd.dv) * std::sqrt(len2(cd.right) * len2(cd.up)) * scale * scale;
+    return area <= 1.0 ? 4 : 8;
+}
+
 // MIP through the brick pass, up to kMaxLaunchCams cameras per pass over the
 // cube: pixel set-up (sample ranges, running maxima, the pass's counters), one staged
 // brick pass, transfer-function finalisation, a launch each for the batch.
@@ -870,7 +895,8 @@ vr_status render_brick_mip(vr_ctx* ctx, float* out_rgba, float* out_max, cudaStr
         pp.zero[1] = static_cast<int*>(ctx->cells);
         VR_CK(launch_pixel_setup(pp, s), "vr_render: pixel set-up");
         if (c0 == 0 && ctx->ev_start) VR_CK(cudaEventRecord(ctx->ev_start, s), "vr_render: profiling event");
-        VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, grid, ctx->cells, s, ctx->tune.group),
+        VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, grid, ctx->cells, s,
+                               pass_group(ctx, ctx->cams[(size_t)c0])),
               "vr_render: brick pass");
         if (c0 + nb >= ncams && ctx->ev_stop) VR_CK(cudaEventRecord(ctx->ev_stop, s), "vr_render: profiling event");
         fp.npix = (long long)nb * img;
@@ -948,7 +974,7 @@ vr_status staged_partials(vr_ctx* ctx, const CamDev& cd, const SortParams& sp, i
     }
     VR_CK(launch_cell_partials(&ctx->tmap_part, bp, sp.tf, ctx->dtype, mode, npartial,
                                cell_partial_passes(ctx->dtype, ctx->B), 2 * ctx->num_sms, ctx->cells, s,
-                               ctx->tune.group),
+                               pass_group(ctx, cd)),
           "sort-last partial images");
     *done = true;
     return VR_OK;
@@ -1260,7 +1286,8 @@ vr_status render_ooc(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
                 bp.work = ctx->work;
                 VR_CK(cudaMemsetAsync(bp.work, 0, sizeof(int), s), "out of core: scheduler reset");
                 VR_CK(cudaMemsetAsync(ctx->cells, 0, sizeof(int), s), "out of core: cell count reset");
-                VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s, ctx->tune.group),
+                VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s,
+                                       pass_group(ctx, cd)),
                       "out of core: brick pass");
             }
             VR_CK(launch_mip_finalize(fp, s), "out of core: finalise");
@@ -1396,7 +1423,8 @@ vr_status brick_mip_with_scratch(vr_ctx* ctx, float* out_rgba, float* out_max, c
         fp.out_max = out_max ? out_max + (long long)i * img : nullptr;
         bp.out_enc = enc;
         VR_CK(launch_pixel_setup(pp, s), "pixel set-up");
-        VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s, ctx->tune.group),
+        VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s,
+                               pass_group(ctx, ctx->cams[(size_t)i])),
               "brick pass");
         VR_CK(launch_mip_finalize(fp, s), "finalise");
     }
@@ -1551,6 +1579,7 @@ vr_status vr_set_tuning(vr_ctx* ctx, const vr_tuning* t) {
         return fail(ctx, VR_ERR_INVALID_ARG,
                     "vr_set_tuning: need tile_w * tile_h == 32, block in {64,128,256}, group in {4,8,16}");
     ctx->tune = *t;
+    ctx->group_set = true;
     return VR_OK;
 }
 
@@ -1565,7 +1594,8 @@ vr_status vr_autotune(vr_ctx* ctx, vr_mode mode, float* scratch_rgba, int reps, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     std::vector<vr_tuning> cands;
     const vr_tuning base = ctx->tune;
-    if (resolve_path(ctx, mode) == VR_PATH_BRICK) {
+    const bool base_set = ctx->group_set, groups = resolve_path(ctx, mode) == VR_PATH_BRICK;
+    if (groups) {
         for (int grp : {4, 8, 16}) cands.push_back(vr_tuning{base.tile_w, base.tile_h, base.block, grp});
     } else {
         const int tiles[5][2] = {{8, 4}, {4, 8}, {16, 2}, {2, 16}, {32, 1}};
@@ -1577,6 +1607,7 @@ vr_status vr_autotune(vr_ctx* ctx, vr_mode mode, float* scratch_rgba, int reps, 
     VR_CK(cudaEventCreate(&e1), "vr_autotune: event");
     const bool saved_graph = ctx->graph_mode;
     ctx->graph_mode = false;
+    ctx->group_set = groups || base_set;  // each candidate as it is
     double best_t = 1e300;
     vr_tuning best_c = base;
     for (const vr_tuning& c : cands) {
@@ -1602,6 +1633,7 @@ vr_status vr_autotune(vr_ctx* ctx, vr_mode mode, float* scratch_rgba, int reps, 
     cudaEventDestroy(e1);
     ctx->graph_mode = saved_graph;
     ctx->tune = (st == VR_OK) ? best_c : base;
+    ctx->group_set = (groups && st == VR_OK) || base_set;
     if (st != VR_OK) return st;
     if (best) *best = best_c;
     if (best_ms) *best_ms = best_t;

@@ -407,10 +407,11 @@ __global__ void k_cell_list(const __grid_constant__ BrickParams P, CellDesc* __r
 }
 
 // One chunk of camera cam's pixel rectangle of a cell -> segment records (phase 1).
-// Records of at most kShortRounds group rounds ("short") fill the chunk's buffer
+// Records of at most short_samples<G>() samples ("short") fill the chunk's buffer
 // from the back, the others from the front, so that the groups of a warp see
 // segments of similar length without a sorting pass.
-constexpr int kShortRounds = 3;
+// (24: with 4 lanes the 25-panel wall takes 49.4 ms, with 12, three rounds of the group, 50.2).
+template <int G> __host__ __device__ constexpr int short_samples() { return G > 8 ? 3 * G : 24; }
 
 template <typename T, bool ONE, int G>
 __device__ __forceinline__ void build_segments(const BrickParams& P, const CamFF& c, int cam_, int4 rect,
@@ -450,7 +451,7 @@ __device__ __forceinline__ void build_segments(const BrickParams& P, const CamFF
         const float4* pd = pd_img ? pd_img + 2 * ((long long)pyv[q] * P.width + pxv[q]) : nullptr;
         if (make_segment<T>(P, c, pxv[q], pyv[q], kr[q], lo, pd, s)) {
             s.pix += (int)(cam * img);
-            if ((s.n & 0x7fffffff) > kShortRounds * G * kUnroll)
+            if ((s.n & 0x7fffffff) > short_samples<G>())
                 segs[atomicAdd(&cnt[0], 1)] = s;
             else
                 segs[kSegCap - 1 - atomicAdd(&cnt[1], 1)] = s;
@@ -688,7 +689,7 @@ template <typename T> struct PartGeom {
 
 // Segment records of one chunk of a cell's pixel rectangle, each pointing at its
 // slot in the partial image of the cell's brick (foot).  Records of at most
-// kShortRounds group rounds fill the buffer from the back, as in the MIP pass.
+// short_samples<G>() samples fill the buffer from the back, as in the MIP pass.
 template <typename T, int G>
 __device__ __forceinline__ void build_part_segments(const BrickParams& P, int4 rect, const BrickFoot& f, float3 lo,
                                                     int c0, SegRec* segs, int* cnt, int tid) {
@@ -721,7 +722,7 @@ __device__ __forceinline__ void build_part_segments(const BrickParams& P, int4 r
         SegRec s;
         if (make_segment<T>(P, c, px, py, kr, lo, pd, s)) {
             s.pix = (int)(f.offset + (long long)(py - f.rect.y) * frw + (px - f.rect.x));
-            if ((s.n & 0x7fffffff) > kShortRounds * G)
+            if ((s.n & 0x7fffffff) > short_samples<G>())
                 segs[atomicAdd(&cnt[0], 1)] = s;
             else
                 segs[kSegCap - 1 - atomicAdd(&cnt[1], 1)] = s;
