@@ -962,7 +962,6 @@ vr_status staged_partials(vr_ctx* ctx, const CamDev& cd, const SortParams& sp, i
     bp.krange = ctx->krange;
     bp.pixdir = ctx->pixdir;  // written by the pixel set-up of this view
     bp.status = ctx->status_dev;
-    bp.work = ctx->work;
     bp.brick_list = brick_list;
     bp.nlist = nlist;
     bp.foot = sp.foot;

@@ -359,6 +359,11 @@ __device__ __forceinline__ bool make_segment(const BrickParams& P, const CamFF& 
     return true;
 }
 
+// The cell-list scratch starts with counters: the cell count of a MIP pass; of the sort-last
+// passes the cells per local key, their fill positions and the passes' work counters.
+constexpr int kCellHeader = 1024;  // bytes
+constexpr int kMaxKeys = 64;       // local keys of a brick: cells per axis <= 8, 8 and 16
+
 struct CellDesc {
     float4 lo;    // lower corner (world voxels); w: the brick id (int bits)
     int4 coord;   // TMA coordinates x, y, z (slot elements), slot
@@ -381,7 +386,6 @@ __global__ void k_cell_list(const __grid_constant__ BrickParams P, CellDesc* __r
         float3 lo;
         int4 coord;
         bool ok = u0 + threadIdx.x < nunits && unit_cell<T>(P, u, lo, coord);
-        if (ok && P.key_pass > 0) ok = cell_key<T>(P, u, coord) == P.key_pass - 1;
         int4 rect0 = make_int4(0, 0, -1, -1);
         if (ok) {
             bool any = cam_cell_rect<T>(P.cams[0], lo, rect0);
@@ -402,6 +406,47 @@ __global__ void k_cell_list(const __grid_constant__ BrickParams P, CellDesc* __r
             d.coord = coord;
             d.rect0 = rect0;
             list[base + __popc(m & ((1u << lane) - 1u))] = d;
+        }
+    }
+}
+
+// The cells of the sort-last passes, grouped by local key: the first launch (SCATTER false)
+// counts them per key, the second writes each key's cells at the sum of the counts before.
+template <typename T, bool SCATTER>
+__global__ void __launch_bounds__(256)
+k_keyed_cells(const __grid_constant__ BrickParams P, CellDesc* __restrict__ list, int* __restrict__ counts,
+              int* __restrict__ fill, int nkeys) {
+    __shared__ int s_first[kMaxKeys];
+    if (SCATTER) {
+        if (threadIdx.x == 0)
+            for (int k = 0, acc = 0; k < nkeys; ++k) {
+                s_first[k] = acc;
+                acc += counts[k];
+            }
+        __syncthreads();
+    }
+    const int ncells = P.ncells_x * P.ncells_y * P.ncells_z;
+    const int nunits = (P.brick_list ? P.nlist : P.nbricks) * ncells;
+    const int lane = threadIdx.x & 31;
+    for (int u0 = blockIdx.x * blockDim.x; u0 < nunits; u0 += gridDim.x * blockDim.x) {
+        int u = u0 + threadIdx.x;
+        if (P.brick_list && u < nunits) u = P.brick_list[u / ncells] * ncells + u % ncells;
+        float3 lo;
+        int4 coord, rect0;
+        const bool ok = u0 + threadIdx.x < nunits && unit_cell<T>(P, u, lo, coord) &&
+                        cam_cell_rect<T>(P.cams[0], lo, rect0);
+        const int key = ok ? cell_key<T>(P, u, coord) : -1;
+        const unsigned int same = __match_any_sync(0xffffffffu, key);
+        const int leader = __ffs(same) - 1;
+        int base = 0;
+        if (ok && lane == leader) base = atomicAdd((SCATTER ? fill : counts) + key, __popc(same));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        if (SCATTER && ok) {
+            CellDesc d;
+            d.lo = make_float4(lo.x, lo.y, lo.z, __int_as_float(u / ncells));
+            d.coord = coord;
+            d.rect0 = rect0;
+            list[s_first[key] + base + __popc(same & ((1u << lane) - 1u))] = d;
         }
     }
 }
@@ -843,12 +888,18 @@ __device__ __forceinline__ void march_part(const BrickParams& P, const T* tile, 
     }
 }
 
-// One pass of the sort-last partials: two CTAs per SM, one staged cell each
-// (the same claim / stage / build pipeline as k_brick_mip, one camera).
+// One pass of the sort-last partials, over the cells of local key `pass` (list: the cells by
+// key, counts: their numbers): two CTAs per SM, one staged cell each (the same claim /
+// stage / build pipeline as k_brick_mip, one camera).  The next pass's CTAs start as this
+// one's leave, stage their first cell and build its segments, and wait for this pass to
+// end only before they touch the slots.  Lists of all keys from two launches and counters
+// from one clear, and this overlap: survey frame PASSES_FIGURES (a list launch, two clears
+// and a drained GPU between any two of the 10 passes before).
 template <typename T, int MODE, int GROUP>
 __global__ void __launch_bounds__(kBrickThreads, 2)
 k_cell_partial(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ BrickParams P,
-               const __grid_constant__ TFDev tf, const CellDesc* __restrict__ list, const int* __restrict__ count) {
+               const __grid_constant__ TFDev tf, const CellDesc* __restrict__ list, const int* __restrict__ counts,
+               int pass) {
     using PG = PartGeom<T>;
     extern __shared__ __align__(128) unsigned char smem[];
     T* tile = reinterpret_cast<T*>(smem);
@@ -862,7 +913,9 @@ k_cell_partial(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
     __shared__ int s_claim[2];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nvalid = *count;
+    grid_launch_dependents();
+    const int nvalid = counts[pass];
+    for (int k = 0; k < pass; ++k) list += counts[k];
     if (MODE == VR_COMPOSITE) fill_table<kMaxPartTF>(s_tf, tf);
     // warp 0: claim the next unit into descriptor slot `slot` (returns the unit)
     auto claim = [&](int slot) {
@@ -904,7 +957,10 @@ k_cell_partial(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
         }
     }
     __syncthreads();
-    if (s_u[0] >= nvalid) return;
+    if (s_u[0] >= nvalid) {
+        grid_wait_before();  // no pass may seem complete before the ones before it are
+        return;
+    }
 
     int cur = 0, chunk = 0, c0 = 0;
     uint32_t phase = 0;
@@ -912,6 +968,7 @@ k_cell_partial(const __grid_constant__ CUtensorMap tmap, const __grid_constant__
     build_part_segments<T, GROUP>(P, s_desc[cur].rect0, s_foot[cur], lo, c0, segs, s_cnt[0], tid);
     bool ok = mbar_wait(&bar, phase, P.status);
     phase ^= 1u;
+    grid_wait_before();  // the slots, and the fill before the first pass
     // a failed wait (2 s without the copy completing) stops the CTA; the next call
     // reports the status (the recovery assumes that the stalled copy never lands)
     if (!__syncthreads_and(ok)) return;
@@ -953,44 +1010,58 @@ __global__ void k_fill_partial(float4* __restrict__ p, long long n, float4 v) {
 
 template <typename T, int MODE, int GROUP>
 cudaError_t launch_part(const void* tmap, const BrickParams& p, const TFDev& tf, int grid, const CellDesc* list,
-                        const int* count, cudaStream_t s) {
+                        const int* counts, int pass, cudaStream_t s) {
     constexpr int SMEM = PartGeom<T>::SMEM;
-    cudaError_t e = cudaFuncSetAttribute(k_cell_partial<T, MODE, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         SMEM);
+    auto* kernel = &k_cell_partial<T, MODE, GROUP>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return e;
-    k_cell_partial<T, MODE, GROUP><<<grid, kBrickThreads, SMEM, s>>>(*static_cast<const CUtensorMap*>(tmap), p, tf,
-                                                                      list, count);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kBrickThreads);
+    cfg.dynamicSmemBytes = SMEM;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = pass > 0 ? 1 : 0;  // the first pass follows the lists and the fill as usual
+    return cudaLaunchKernelEx(&cfg, kernel, *static_cast<const CUtensorMap*>(tmap), p, tf, list, counts, pass);
 }
 
 template <typename T>
 cudaError_t cell_partials_t(const void* tmap, const BrickParams& p0, const TFDev& tf, int mode, long long npartial,
                             int npass, int grid, void* cells, cudaStream_t s, int group) {
-    CellDesc* list = reinterpret_cast<CellDesc*>(static_cast<char*>(cells) + 256);
-    int* count = static_cast<int*>(cells);
+    if (npass > kMaxKeys) return cudaErrorInvalidValue;
+    CellDesc* list = reinterpret_cast<CellDesc*>(static_cast<char*>(cells) + kCellHeader);
+    int* counts = static_cast<int*>(cells);
+    int *fill = counts + kMaxKeys, *work = fill + kMaxKeys;
+    static_assert(3 * kMaxKeys * sizeof(int) <= kCellHeader, "counters fit the header");
     const float4 empty = mode == VR_MIP ? make_float4(-INFINITY, 0.f, 0.f, 0.f) : make_float4(0.f, 0.f, 0.f, 1.f);
+    cudaError_t e = cudaMemsetAsync(cells, 0, kCellHeader, s);
+    if (e != cudaSuccess) return e;
+    BrickParams p = p0;
+    const int nunits = (p.brick_list ? p.nlist : p.nbricks) * p.ncells_x * p.ncells_y * p.ncells_z;
+    const int blocks = std::min((nunits + 255) / 256, 4096);
+    k_keyed_cells<T, false><<<blocks, 256, 0, s>>>(p, list, counts, fill, npass);
+    k_keyed_cells<T, true><<<blocks, 256, 0, s>>>(p, list, counts, fill, npass);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     if (npartial > 0) {
         k_fill_partial<<<(int)std::min<long long>((npartial + 255) / 256, 152 * 16), 256, 0, s>>>(p0.partial,
                                                                                                   npartial, empty);
-        cudaError_t e = cudaGetLastError();
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    BrickParams p = p0;
-    const int nunits = (p.brick_list ? p.nlist : p.nbricks) * p.ncells_x * p.ncells_y * p.ncells_z;
     for (int pass = 0; pass < npass; ++pass) {
-        p.key_pass = pass + 1;
-        cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p.work, 0, sizeof(int), s);
-        if (e != cudaSuccess) return e;
-        k_cell_list<T><<<std::min((nunits + 255) / 256, 4096), 256, 0, s>>>(p, list, count);
+        p.work = work + pass;
         if (mode == VR_MIP)
-            e = group == 4    ? launch_part<T, VR_MIP, 4>(tmap, p, tf, grid, list, count, s)
-                : group == 16 ? launch_part<T, VR_MIP, 16>(tmap, p, tf, grid, list, count, s)
-                              : launch_part<T, VR_MIP, 8>(tmap, p, tf, grid, list, count, s);
+            e = group == 4    ? launch_part<T, VR_MIP, 4>(tmap, p, tf, grid, list, counts, pass, s)
+                : group == 16 ? launch_part<T, VR_MIP, 16>(tmap, p, tf, grid, list, counts, pass, s)
+                              : launch_part<T, VR_MIP, 8>(tmap, p, tf, grid, list, counts, pass, s);
         else
-            e = group == 4    ? launch_part<T, VR_COMPOSITE, 4>(tmap, p, tf, grid, list, count, s)
-                : group == 16 ? launch_part<T, VR_COMPOSITE, 16>(tmap, p, tf, grid, list, count, s)
-                              : launch_part<T, VR_COMPOSITE, 8>(tmap, p, tf, grid, list, count, s);
+            e = group == 4    ? launch_part<T, VR_COMPOSITE, 4>(tmap, p, tf, grid, list, counts, pass, s)
+                : group == 16 ? launch_part<T, VR_COMPOSITE, 16>(tmap, p, tf, grid, list, counts, pass, s)
+                              : launch_part<T, VR_COMPOSITE, 8>(tmap, p, tf, grid, list, counts, pass, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1050,7 +1121,7 @@ cudaError_t launch_brick_g(const void* tmap, const BrickParams& p, int grid, con
 
 template <typename T>
 cudaError_t launch_t(const void* tmap, const BrickParams& p, int grid, void* cells, cudaStream_t s, int group) {
-    CellDesc* list = reinterpret_cast<CellDesc*>(static_cast<char*>(cells) + 256);
+    CellDesc* list = reinterpret_cast<CellDesc*>(static_cast<char*>(cells) + kCellHeader);
     int* count = static_cast<int*>(cells);
     const int nunits = (p.brick_list ? p.nlist : p.nbricks) * p.ncells_x * p.ncells_y * p.ncells_z;
     k_cell_list<T><<<std::min((nunits + 255) / 256, 4096), 256, 0, s>>>(p, list, count);
@@ -1105,7 +1176,7 @@ int cell_partial_passes(vr_dtype dt, int brick) {
 
 cudaError_t launch_cell_partials(const void* tmap, const BrickParams& p, const TFDev& tf, vr_dtype dt, int mode,
                                  long long npartial, int npass, int grid, void* cells, cudaStream_t s, int group) {
-    if (tf.n > kMaxPartTF || !p.partial || !p.foot || !p.work) return cudaErrorInvalidValue;
+    if (tf.n > kMaxPartTF || !p.partial || !p.foot) return cudaErrorInvalidValue;
     if (dt == VR_F32) return cell_partials_t<float>(tmap, p, tf, mode, npartial, npass, grid, cells, s, group);
     if (dt == VR_F16) return cell_partials_t<__half>(tmap, p, tf, mode, npartial, npass, grid, cells, s, group);
     return cell_partials_t<__nv_bfloat16>(tmap, p, tf, mode, npartial, npass, grid, cells, s, group);
@@ -1124,7 +1195,7 @@ cudaError_t launch_mip_finalize(const FinalizeParams& p, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-size_t brick_cells_bytes(long long nunits) { return 256 + (size_t)nunits * sizeof(CellDesc); }
+size_t brick_cells_bytes(long long nunits) { return kCellHeader + (size_t)nunits * sizeof(CellDesc); }
 
 cudaError_t launch_brick_mip(const void* tmap, const BrickParams& p, vr_dtype dt, int grid, void* cells,
                              cudaStream_t s, int group) {

@@ -109,7 +109,6 @@ struct BrickParams {
     // with the same key, so the cells of a pass fold into disjoint pixels.
     const BrickFoot* foot;   // per brick: rectangle and offset of its partial image
     float4* partial;         // partial images: (C, T), or the maximum in .x (MIP)
-    int key_pass;            // k_cell_list keeps the cells of local key key_pass - 1 only (0: all cells)
     int key_persp;           // 1: perspective key, 0: orthographic key
     int eye_cell[3];         // perspective: floor(eye / cell edge) per axis, clamped
     int key_sign[3];         // orthographic: sign of the view direction per axis

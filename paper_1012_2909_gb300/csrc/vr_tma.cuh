@@ -76,6 +76,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
     return false;
 }
 
+// Programmatic dependent launch: let the next launch of the stream start its prologue, and
+// wait in a prologue until the launches before it are complete and their writes visible.
+__device__ __forceinline__ void grid_launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_wait_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // 4-D tiled TMA load of a box into shared memory, completing on `bar`.
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar,
                                             int c0, int c1, int c2, int c3) {
