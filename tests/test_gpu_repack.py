@@ -37,3 +37,27 @@ def test_store_from_device_and_host(storage, brick, dims):
                     compare(got[1][i].reshape(-1, 4), sc, c, "mip", tol=1e-4)
             for a, b in zip(ref, got):
                 np.testing.assert_array_equal(a, b)
+
+
+def test_replaced_cubes_equal_fresh_ones():
+    """A renderer that loads cube after cube, with and without taking over the buffers (the same
+    bricks, or another size or type width), against a fresh renderer for each."""
+    import paper_1012_2909_gb300 as vr
+    tf = synth.viridis_ramp_tf()
+    kept = vr.Renderer(0, brick=64)
+    for i, (dims, storage, host) in enumerate((((90, 70, 65), "f16", False), ((100, 66, 128), "bf16", False),
+                                               ((100, 66, 128), "f32", False), ((90, 70, 65), "f32", True),
+                                               ((90, 70, 60), "f16", True), ((90, 70, 65), "f16", False))):
+        vol = synth.generate(synth.cube_params(*dims, seed=40 + i, nsrc=5))
+        src = vol if host else torch.from_numpy(vol).cuda()
+        got = []
+        for r in (kept, vr.Renderer(0, brick=64)):
+            r.load_cube(src, storage)
+            r.set_transfer_function(tf, -1.0, 20.0)
+            r.set_camera(synth.look_at(dims, (0.4, 0.3, 1.0), 45, 27))
+            for mode, path in (("composite", "ray"), ("composite", "layered"), ("composite", "sortlast"), ("mip", "brick")):
+                r.set_path(path)
+                got.append(r.render(mode).cpu().numpy())
+            assert r.cube_info()["nx"] == dims[0] and r.cube_info()["nz"] == dims[2]
+        for a, b in zip(got[:4], got[4:]):
+            np.testing.assert_array_equal(a, b)
