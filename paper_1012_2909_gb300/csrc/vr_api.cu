@@ -824,6 +824,19 @@ FinalizeParams finalize_params(const vr_ctx* ctx) {
     return p;
 }
 
+// Area of a pixel, in square voxels, at the cube's centre.
+double pixel_area(const vr_ctx* ctx, const CamDev& cd) {
+    const double c[3] = {0.5 * (double)ctx->nx, 0.5 * (double)ctx->ny, 0.5 * (double)ctx->nz};
+    auto len2 = [](const double* v) { return v[0] * v[0] + v[1] * v[1] + v[2] * v[2]; };
+    double scale = 1.0;  // of the window at the cube's centre
+    if (cd.type == 1) {
+        scale = 0.0;
+        for (int a = 0; a < 3; ++a) scale += (c[a] - cd.eye[a]) * cd.fwd[a];
+        scale = std::fabs(scale) / len2(cd.fwd);
+    }
+    return std::fabs(cd.du * cd.dv) * std::sqrt(len2(cd.right) * len2(cd.up)) * scale * scale;
+}
+
 // Lanes per ray segment of a staged-cell pass over views like `cd`: the tuning's where the
 // caller or the autotuner set one, else by the length of the segments and the spacing of
 // the rays at the cube's centre.  Fewer lanes waste less on a segment's last step, and pay
@@ -836,16 +849,14 @@ FinalizeParams finalize_params(const vr_ctx* ctx) {
 int pass_group(const vr_ctx* ctx, const CamDev& cd) {
     if (ctx->group_set) return ctx->tune.group;
     if (ctx->dtype == VR_F32) return 4;
-    const double c[3] = {0.5 * (double)ctx->nx, 0.5 * (double)ctx->ny, 0.5 * (double)ctx->nz};
-    auto len2 = [](const double* v) { return v[0] * v[0] + v[1] * v[1] + v[2] * v[2]; };
-    double scale = 1.0;  // of the window at the cube's centre
-    if (cd.type == 1) {
-        scale = 0.0;
-        for (int a = 0; a < 3; ++a) scale += (c[a] - cd.eye[a]) * cd.fwd[a];
-        scale = std::fabs(scale) / len2(cd.fwd);
-    }
-    const double area = std::fabs(cd.du * cd.dv) * std::sqrt(len2(cd.right) * len2(cd.up)) * scale * scale;
-    return area <= 1.0 ? 4 : 8;
+    return pixel_area(ctx, cd) <= 1.0 ? 4 : 8;
+}
+
+// Most row bands of a staged cell's pixels (BrickParams::max_bands): a 32^3 cell covers
+// some 1500 square voxels, and a band should keep 512 pixels.
+int pass_bands(const vr_ctx* ctx, const CamDev& cd) {
+    const double px = 1500.0 / std::max(pixel_area(ctx, cd), 1e-3);
+    return (int)std::min(64.0, std::max(1.0, px / 512.0));
 }
 
 // MIP through the brick pass, up to kMaxLaunchCams cameras per pass over the
@@ -888,6 +899,7 @@ vr_status render_brick_mip(vr_ctx* ctx, float* out_rgba, float* out_max, cudaStr
             pp.cams[i] = bp.cams[i];
         }
         bp.out_enc = enc;
+        bp.max_bands = pass_bands(ctx, ctx->cams[(size_t)c0]);
         bp.work = ctx->work + kMaxLaunchCams + (c0 / per) % 4096;
         pp.ncams = nb;
         pp.enc = enc;
@@ -964,6 +976,7 @@ vr_status staged_partials(vr_ctx* ctx, const CamDev& cd, const SortParams& sp, i
     bp.status = ctx->status_dev;
     bp.brick_list = brick_list;
     bp.nlist = nlist;
+    bp.max_bands = pass_bands(ctx, cd);
     bp.foot = sp.foot;
     bp.partial = sp.partial;
     bp.key_persp = cd.type == 1;
@@ -1421,6 +1434,7 @@ vr_status brick_mip_with_scratch(vr_ctx* ctx, float* out_rgba, float* out_max, c
         fp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)i * img;
         fp.out_max = out_max ? out_max + (long long)i * img : nullptr;
         bp.out_enc = enc;
+        bp.max_bands = pass_bands(ctx, ctx->cams[(size_t)i]);
         VR_CK(launch_pixel_setup(pp, s), "pixel set-up");
         VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s,
                                pass_group(ctx, ctx->cams[(size_t)i])),

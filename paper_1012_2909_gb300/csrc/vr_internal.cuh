@@ -91,7 +91,8 @@ struct BrickParams {
     int ncams, width, height;
     float step, step_lo;     // the sample spacing as a float-float pair
     int ncells_x, ncells_y, ncells_z;  // cells per brick along each axis
-    int nbricks, pad_b;
+    int nbricks;
+    int max_bands;           // most row bands a cell's pixels may be split into (0 or 1: none)
     const int2* krange;      // per pixel [k0, k1) from the pixel set-up
     const float4* pixdir;    // optional, perspective cameras: per pixel the step
                              // vector e in float-float, 2 x float4 (hi.xyz, lo.x),
