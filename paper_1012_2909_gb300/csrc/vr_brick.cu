@@ -34,13 +34,15 @@ static_assert(kSegCap % kBrickThreads == 0, "segment chunk must be a multiple of
 constexpr int kUnroll = 1;  // samples per lane per step (2 measured no faster)
 
 // Staged cell: CX x CY x CZ interior voxels, TMA box BX x BY x BZ (ghost
-// included, x padded to 16 bytes).  The 16-bit box has one spare row (BY = 35,
-// never read back): the slab stride becomes 700 words, 28 banks apart instead
-// of 8, which spreads the gathers of neighbouring z-slabs over the banks
-// (1 % faster over the survey orbit; the largest box that keeps two CTAs per SM).
+// included, x padded to 16 bytes).  The boxes have spare rows (never read back) that
+// spread the gathers of neighbouring z-slabs over the banks: one in the 16-bit box
+// (BY = 35, a slab stride of 700 words, 28 banks apart instead of 8: 1 % faster over the
+// survey orbit), three in the FP32 box (BY = 37, 1332 words, 20 banks apart instead of 8:
+// 1721 x 1721 x 1025 at 3000 x 3000 18.91 -> 18.69 ms, with one row 18.88).  They are the
+// largest boxes that keep two CTAs per SM.
 template <typename T> struct Cell;
 template <> struct Cell<float> {
-    static constexpr int CX = 32, CY = 32, CZ = 16, BX = 36, BY = 34, BZ = 18;
+    static constexpr int CX = 32, CY = 32, CZ = 16, BX = 36, BY = 37, BZ = 18;
 };
 template <> struct Cell<__half> {
     static constexpr int CX = 32, CY = 32, CZ = 32, BX = 40, BY = 35, BZ = 34;
@@ -743,7 +745,7 @@ k_brick_mip(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ Br
 // segment with G lanes on consecutive samples, and folds the segment into the brick's slot: C += T C_seg, T *= T_seg
 // (or the maximum).  Slots start as the empty image (0, 0, 0, 1), or -inf.
 
-// Staged box without the spare row (the partial pass also holds the table).
+// Staged box without spare rows (the partial pass also holds the table).
 template <typename T> struct PartGeom {
     static constexpr int BY = Cell<T>::CY + 2;
     static constexpr int BYTES = Cell<T>::BX * BY * Cell<T>::BZ * (int)sizeof(T);

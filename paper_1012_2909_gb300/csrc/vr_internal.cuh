@@ -223,13 +223,13 @@ cudaError_t launch_cell_partials(const void* tmap, const BrickParams& p, const T
                                  int group = 8);
 // Number of visibility passes launch_cell_partials needs for a brick edge.
 int cell_partial_passes(vr_dtype dt, int brick);
-// TMA box of one cell for launch_cell_partials (no spare row), in elements.
+// TMA box of one cell for launch_cell_partials (no spare rows), in elements.
 void brick_part_box_dims(vr_dtype dt, int* bx, int* by, int* bz);
 // Cell (staging unit) edge lengths for a storage type; the brick edge must be a
 // multiple of each.
 void brick_cell_dims(vr_dtype dt, int* cx, int* cy, int* cz);
-// TMA box of one cell (cell + 2 ghost, x padded to 16 bytes, one spare row for
-// 16-bit stores), in elements.
+// TMA box of one cell (cell + 2 ghost, x padded to 16 bytes, spare rows), in
+// elements.
 void brick_box_dims(vr_dtype dt, int* bx, int* by, int* bz);
 // Footprints, keys and the visibility order of the bricks (p.order, p.layer_*).
 cudaError_t launch_brick_footprints(const SortParams& p, cudaStream_t s);
