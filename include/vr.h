@@ -240,7 +240,7 @@ vr_status vr_render_backward(vr_ctx* ctx, vr_mode mode, const float* dL_dimg, fl
  *   group:           lanes per ray segment in the brick path (4, 8, 16), i.e.
  *                    32 / group rays per warp.
  * Defaults 8 x 4, 256, 8; until a tuning is set, the brick path takes 4 lanes
- * instead for FP32 cells and for views whose rays are dense.  Results do not
+ * instead where the rays are dense (with FP32 cells also where less so).  Results do not
  * depend on the tuning (up to rounding). */
 typedef struct {
     int32_t tile_w, tile_h;
