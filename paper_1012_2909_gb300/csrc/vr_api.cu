@@ -843,9 +843,9 @@ double pixel_area(const vr_ctx* ctx, const CamDev& cd) {
 // where neighbouring groups march segments of one length: in the short segments of FP32
 // cells (16 voxels thick: 1721 x 1721 x 1025 at 1.0 voxels a pixel 18.9 ms with 4 lanes and
 // 19.7 with 8; equal within 1 % up to 3 voxels a pixel; 1269 x 339 x 736 at 7.8 voxels a
-// pixel 0.313 and 0.301; not measured between), and with 16-bit cells where the rays are at most a voxel apart
-// (2048 x 2048 x 1024 on 25 panels: 0.66 voxels 49.4 and 53.3 ms, 0.99 25.6 and 26.0;
-// 1.31 16.6 and 16.3; 1024 x 1024 x 2048 at 2.7 voxels 2.57 and 2.27).
+// pixel 0.313 and 0.301; not measured between), and with 16-bit cells where the rays are
+// at most a voxel apart (2048 x 2048 x 1024 on 25 panels: 0.66 voxels 49.4 and
+// 53.3 ms, 0.99 25.6 and 26.0; 1.31 16.6 and 16.3; 1024 x 1024 x 2048 at 2.7 voxels 2.57 and 2.27).
 int pass_group(const vr_ctx* ctx, const CamDev& cd) {
     if (ctx->group_set) return ctx->tune.group;
     return pixel_area(ctx, cd) <= (ctx->dtype == VR_F32 ? 9.0 : 1.0) ? 4 : 8;
