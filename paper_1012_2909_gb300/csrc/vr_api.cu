@@ -61,6 +61,8 @@ struct vr_ctx {
     bool has_tf = false;
     std::vector<float4> tf;
     float vmin = 0.f, vmax = 1.f;
+    bool tf_steep = false;         // neighbouring entries further apart than FP32 reaches
+    double tf_growth = 1.0;        // largest |1 - opacity|
     // cameras
     std::vector<CamDev> cams;
     // brick pass: TMA descriptor of the brick store
@@ -620,6 +622,14 @@ vr_status vr_set_transfer_function(vr_ctx* ctx, const float* rgba, int n, float 
             if (!std::isfinite(rgba[4 * i + c]))
                 return fail(ctx, VR_ERR_INVALID_ARG, "vr_set_transfer_function: non-finite entry");
     }
+    ctx->tf_steep = false;
+    ctx->tf_growth = 0.0;
+    for (int i = 0; i < n; ++i) {
+        const float4 a = t[(size_t)i], b = t[(size_t)std::min(i + 1, n - 1)];
+        ctx->tf_steep |= !std::isfinite(b.x - a.x) || !std::isfinite(b.y - a.y) || !std::isfinite(b.z - a.z) ||
+                         !std::isfinite(b.w - a.w);
+        ctx->tf_growth = std::max(ctx->tf_growth, std::fabs(1.0 - (double)a.w));
+    }
     ctx->tf.swap(t);
     ctx->vmin = vmin;
     ctx->vmax = vmax;
@@ -744,6 +754,14 @@ TFDev tf_dev(const vr_ctx* ctx) {
     return t;
 }
 
+// Whether a composite may meet values beyond FP32: a lookup between entries too far apart, or
+// a transmittance grown by opacities outside [0, 1] over the samples of the longest ray.
+bool march_guard(const vr_ctx* ctx) {
+    const double d2 = (double)ctx->nx * ctx->nx + (double)ctx->ny * ctx->ny + (double)ctx->nz * ctx->nz;
+    return ctx->tf_steep ||
+           (ctx->tf_growth > 1.0 && std::log(ctx->tf_growth) * (std::sqrt(d2) / ctx->opt.step + 2.0) > 88.0);
+}
+
 // Image order: the marcher, or (layered, composite only) its form that walks the bricks
 // as parts with carried state.
 vr_status render_ray(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max, cudaStream_t s,
@@ -765,6 +783,7 @@ vr_status render_ray(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
     split(ctx->opt.step, P.step_hi, P.step_lo);
     P.ert = (float)ctx->opt.ert;
     P.samples = ctx->sample_counter;
+    P.guard = mode == VR_COMPOSITE && march_guard(ctx);
     const int block = ctx->tune.block;
     const int per_sm = layered ? layered_blocks_per_sm(P, ctx->dtype, block) : march_blocks_per_sm(P, ctx->dtype, block);
     const int grid = ctx->num_sms * per_sm * block / 32;

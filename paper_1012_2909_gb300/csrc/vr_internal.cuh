@@ -72,7 +72,7 @@ struct MarchParams {
     int tile_w, tile_h;          // pixels of one warp work item (tile_w * tile_h == 32)
     float step_hi, step_lo;      // the sample spacing as a float-float pair
     float ert;
-    int pad2;
+    int guard;                   // a lookup or a transmittance may leave FP32's range
     float4* out_rgba;            // pixels of camera 0 of this launch
     float* out_max;              // may be null
     unsigned long long* samples; // may be null
@@ -190,6 +190,17 @@ struct FinalizeParams {
     float4* out_rgba;
     float* out_max;  // may be null, or enc itself
 };
+
+// Forms of the per-ray composites: the default brick edge and small tables compiled in; any
+// brick and table; the same, with samples past a ray's end passed over by a branch instead of
+// composited with opacity 0 (where 0 times a value beyond FP32 would not be 0).  The branch
+// for every table would cost the 128^3 FP32 view 66.2 -> 71.7 us and the survey frame 333 ->
+// 354 us, so only tables that can reach such values take it.
+enum MarchForm { kFormFast, kFormGeneral, kFormGuarded };
+inline MarchForm march_form(const MarchParams& p, int table) {
+    if (p.guard) return kFormGuarded;
+    return p.vol.B == kFastBrick && p.tf.n <= table ? kFormFast : kFormGeneral;
+}
 
 // Host-side launchers (defined in the kernel translation units).
 // Brick layers [bz0, bz0 + nlayers) of the store (and of its copy shifted by one element,

@@ -26,7 +26,7 @@ constexpr int kMarchUnroll = 4;
 constexpr int kMarchUnrollPaired = 6;
 
 // Tables of up to kMarchTF entries are kept with the rises of their intervals, and the
-// default brick edge is compiled in (FAST); other tables and edges take the general form.
+// default brick edge is compiled in (kFormFast); other tables and edges take the general form.
 //
 // Bound by L1 wavefronts on sparse views (profile: 72-79 %) and by the instructions of 16
 // warps an SM on dense ones: a sample took about 130 warp instructions on the small FP32
@@ -55,9 +55,10 @@ __device__ __forceinline__ void prefetch_near(const T* slot, const T* slot1, con
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p + SlotGeom<T, BR>::slab(v)));
 }
 
-template <typename T, int MODE, bool PAIRED, bool FAST>
+template <typename T, int MODE, bool PAIRED, MarchForm FORM>
 __global__ void __launch_bounds__(256, 2)
 k_march(const __grid_constant__ MarchParams P) {
+    constexpr bool FAST = FORM == kFormFast;
     constexpr int U = PAIRED ? kMarchUnrollPaired : kMarchUnroll;
     constexpr int BR = FAST ? kFastBrick : 0, S = FAST ? kMarchTF : kMaxTF;
     __shared__ float s_tf[(FAST ? 8 : 4) * S];
@@ -125,6 +126,7 @@ k_march(const __grid_constant__ MarchParams P) {
                             } else {
                                 // past the span or the termination: opacity 0, nothing changes
                                 const bool on = i + q < m && !done;
+                                if (FORM == kFormGuarded && !on) break;
                                 const float4 c = tf_lookup<S, FAST>(s_tf, P.tf.n, P.tf.vmin, P.tf.inv_range, v[q]);
                                 const float a = on ? c.w : 0.f;
                                 const float w = Tr * a;
@@ -163,28 +165,31 @@ k_march(const __grid_constant__ MarchParams P) {
 }
 
 template <typename T, int MODE, bool PAIRED>
-void* kernel_ptr(bool fast) {
-    return fast ? reinterpret_cast<void*>(&k_march<T, MODE, PAIRED, true>)
-                : reinterpret_cast<void*>(&k_march<T, MODE, PAIRED, false>);
+void* kernel_ptr(MarchForm form) {
+    if (MODE == VR_COMPOSITE && form == kFormGuarded)
+        return reinterpret_cast<void*>(&k_march<T, VR_COMPOSITE, PAIRED, kFormGuarded>);
+    return form == kFormFast ? reinterpret_cast<void*>(&k_march<T, MODE, PAIRED, kFormFast>)
+                             : reinterpret_cast<void*>(&k_march<T, MODE, PAIRED, kFormGeneral>);
 }
 
 // Paired loads only for the composite: its rays stop in a front shell that stays in
 // the caches, where halving the gathers pays (survey frame -11 %).  MIP rays cross the
 // whole cube, and reading both copies there measured 34 % slower.
 template <typename T>
-void* pick_mode(int mode, bool paired, bool fast) {
-    if (mode == VR_MIP) return kernel_ptr<T, VR_MIP, false>(fast);
+void* pick_mode(int mode, bool paired, MarchForm form) {
+    if (mode == VR_MIP) return kernel_ptr<T, VR_MIP, false>(form);
     if constexpr (sizeof(T) == 2) {
-        if (paired) return kernel_ptr<T, VR_COMPOSITE, true>(fast);
+        if (paired) return kernel_ptr<T, VR_COMPOSITE, true>(form);
     }
-    return kernel_ptr<T, VR_COMPOSITE, false>(fast);
+    return kernel_ptr<T, VR_COMPOSITE, false>(form);
 }
 
 void* pick(vr_dtype dt, const MarchParams& p) {
-    const bool paired = p.vol.pool1 != nullptr, fast = p.vol.B == kFastBrick && p.tf.n <= kMarchTF;
-    if (dt == VR_F32) return pick_mode<float>(p.mode, paired, fast);
-    if (dt == VR_F16) return pick_mode<__half>(p.mode, paired, fast);
-    return pick_mode<__nv_bfloat16>(p.mode, paired, fast);
+    const bool paired = p.vol.pool1 != nullptr;
+    const MarchForm form = march_form(p, kMarchTF);
+    if (dt == VR_F32) return pick_mode<float>(p.mode, paired, form);
+    if (dt == VR_F16) return pick_mode<__half>(p.mode, paired, form);
+    return pick_mode<__nv_bfloat16>(p.mode, paired, form);
 }
 
 }  // namespace

@@ -383,14 +383,15 @@ k_brick_partial(const __grid_constant__ SortParams P, int layer_begin, int layer
 // loads U = 4, 5, 6 take 0.475, 0.456, 0.464 ms.
 constexpr int kLayeredUnroll = 4;
 constexpr int kLayeredUnrollPaired = 5;
-constexpr int kLayeredTF = 256;  // FAST: the default brick edge and tables up to this size, as in k_march
+constexpr int kLayeredTF = 256;  // kFormFast: the default brick edge and tables up to this size, as in k_march
 
 // One brick's samples [0, n) at slot coordinates g + j e, composited onto (C, Tr); true
 // once 1 - Tr reaches ert.  CLAMP keeps the coordinates inside the slot.
-template <typename T, bool PAIRED, bool FAST, bool CLAMP>
+template <typename T, bool PAIRED, MarchForm FORM, bool CLAMP>
 __device__ __forceinline__ bool layered_walk(const T* slot, const T* slot1, const VolDev& v, const TFDev& tf,
                                              const float* s_tf, float3 g, float3 e, int n, float ert, float& C0,
                                              float& C1, float& C2, float& Tr) {
+    constexpr bool FAST = FORM == kFormFast;
     constexpr int U = PAIRED ? kLayeredUnrollPaired : kLayeredUnroll;
     constexpr int BR = FAST ? kFastBrick : 0, S = FAST ? kLayeredTF : kMaxTF;
     const Anchor A{0.f, 0.f, 0.f, 0};  // offsets from the slot's first voxel
@@ -413,6 +414,7 @@ __device__ __forceinline__ bool layered_walk(const T* slot, const T* slot1, cons
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const bool on = i + q < n && !done;  // else opacity 0: nothing changes
+            if (FORM == kFormGuarded && !on) break;
             const float4 t = tf_lookup<S, FAST>(s_tf, tf.n, tf.vmin, tf.inv_range, val[q]);
             const float a = on ? t.w : 0.f;
             const float w = Tr * a;
@@ -426,9 +428,10 @@ __device__ __forceinline__ bool layered_walk(const T* slot, const T* slot1, cons
     return done;
 }
 
-template <typename T, bool PAIRED, bool FAST>
+template <typename T, bool PAIRED, MarchForm FORM>
 __global__ void __launch_bounds__(256, 2)
 k_march_layered(const __grid_constant__ MarchParams P) {
+    constexpr bool FAST = FORM == kFormFast;
     constexpr int S = FAST ? kLayeredTF : kMaxTF;
     __shared__ float s_tf[(FAST ? 8 : 4) * S];
     fill_table<S, FAST>(s_tf, P.tf);
@@ -509,9 +512,9 @@ k_march_layered(const __grid_constant__ MarchParams P) {
                     const float x1 = fmaf(fl, e32.x, g.x), y1 = fmaf(fl, e32.y, g.y), z1 = fmaf(fl, e32.z, g.z);
                     const bool inside = fminf(fminf(fminf(g.x, x1), fminf(g.y, y1)), fminf(g.z, z1)) >= 0.f &&
                                         fmaxf(fmaxf(fmaxf(g.x, x1), fmaxf(g.y, y1)), fmaxf(g.z, z1)) <= hi;
-                    done = inside ? layered_walk<T, PAIRED, FAST, false>(slot, slot1, P.vol, P.tf, s_tf, g, e32, n, ert,
+                    done = inside ? layered_walk<T, PAIRED, FORM, false>(slot, slot1, P.vol, P.tf, s_tf, g, e32, n, ert,
                                                                          C0, C1, C2, Tr)
-                                  : layered_walk<T, PAIRED, FAST, true>(slot, slot1, P.vol, P.tf, s_tf, g, e32, n, ert,
+                                  : layered_walk<T, PAIRED, FORM, true>(slot, slot1, P.vol, P.tf, s_tf, g, e32, n, ert,
                                                                         C0, C1, C2, Tr);
                 }
                 k = kb;
@@ -646,21 +649,26 @@ cudaError_t launch_brick_partial(const SortParams& p, vr_dtype dt, bool carried,
 }
 
 namespace {
+template <typename T, bool PAIRED>
+void* layered_form(MarchForm form) {
+    if (form == kFormGuarded) return reinterpret_cast<void*>(&k_march_layered<T, PAIRED, kFormGuarded>);
+    return form == kFormFast ? reinterpret_cast<void*>(&k_march_layered<T, PAIRED, kFormFast>)
+                             : reinterpret_cast<void*>(&k_march_layered<T, PAIRED, kFormGeneral>);
+}
+
 template <typename T>
-void* layered_t(bool paired, bool fast) {
+void* layered_t(bool paired, MarchForm form) {
     if constexpr (sizeof(T) == 2) {
-        if (paired)
-            return fast ? reinterpret_cast<void*>(&k_march_layered<T, true, true>)
-                        : reinterpret_cast<void*>(&k_march_layered<T, true, false>);
+        if (paired) return layered_form<T, true>(form);
     }
-    return fast ? reinterpret_cast<void*>(&k_march_layered<T, false, true>)
-                : reinterpret_cast<void*>(&k_march_layered<T, false, false>);
+    return layered_form<T, false>(form);
 }
 
 void* layered_ptr(vr_dtype dt, const MarchParams& p) {
-    const bool paired = p.vol.pool1 != nullptr, fast = p.vol.B == kFastBrick && p.tf.n <= kLayeredTF;
-    if (dt == VR_F32) return layered_t<float>(paired, fast);
-    return dt == VR_F16 ? layered_t<__half>(paired, fast) : layered_t<__nv_bfloat16>(paired, fast);
+    const bool paired = p.vol.pool1 != nullptr;
+    const MarchForm form = march_form(p, kLayeredTF);
+    if (dt == VR_F32) return layered_t<float>(paired, form);
+    return dt == VR_F16 ? layered_t<__half>(paired, form) : layered_t<__nv_bfloat16>(paired, form);
 }
 }  // namespace
 
