@@ -106,7 +106,9 @@ k_repack(const float* __restrict__ src, long long src_z0, int bz0, VolDev v, T* 
         float f[U][VPW], f2[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const float* row = plane + (long long)min(max(y0 + ly0 + u * lines, 0), v.ny - 1) * v.nx;
+            // rows past the slot's last one repeat it
+            const int ly = min(ly0 + u * lines, v.rows - 1);
+            const float* row = plane + (long long)min(max(y0 + ly, 0), v.ny - 1) * v.nx;
             f[u][0] = real ? __ldg(row + c0) : 0.f;
             if (VPW == 2) f[u][VPW - 1] = real ? __ldg(row + c1) : 0.f;
             f2[u] = third ? __ldg(row + c2) : 0.f;
@@ -117,7 +119,7 @@ k_repack(const float* __restrict__ src, long long src_z0, int bz0, VolDev v, T* 
             const bool put = mine && ly < v.rows;
             if constexpr (VPW == 2) {
                 const T a = to_store<T>(f[u][0]), b = to_store<T>(f[u][1]);
-                if (real) range.add(a, b);  // rows past the last repeat it
+                if (real) range.add(a, b);  // a repeated row adds nothing new
                 const unsigned int lo = bits(a), hi = bits(b);
                 if (put) dst[ly * row_words + word] = lo | (hi << 16);
                 if (COPY) {
