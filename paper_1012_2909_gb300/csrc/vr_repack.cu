@@ -67,7 +67,10 @@ template <> struct Range<float> {
 // down the plane in that column, so its clamped source columns are found once and a
 // word costs few instructions.  Loads and stores of a warp are consecutive words
 // whatever the source's alignment (a row starts one voxel before the brick, so wider
-// loads would never be aligned); kRepackUnroll rows' loads are in flight.  The copy's
+// loads would never be aligned); kRepackUnroll rows' loads are in flight, and the rows of
+// threads in a block are chosen so that its trips end near the slot's last row (blocks of
+// kRepackThreads whatever the brick went far past it in small ones: 512^3 FP16 in bricks of
+// 8, 16, 32, 64 voxels 7.9, 1.86, 0.51, 0.29 ms a load, now 1.36, 0.49, 0.38, 0.26).  The copy's
 // word (voxels x + 1, x + 2) is made from the same registers and the next lane's, in
 // place of a device-to-device copy at a 2-byte offset afterwards.  Neighbouring bricks
 // read the ghost planes and row ends again, so the loads go through L2 as usual: with
@@ -149,7 +152,10 @@ cudaError_t repack_t(const float* src, long long src_z0, int bz0, int nlayers, c
                      void* pool1, unsigned int* minmax, cudaStream_t s) {
     const int nbricks = v.nbx * v.nby * v.nbz;
     const int row_words = v.pitch * (int)sizeof(T) / 4;  // 8 .. 260
-    const int lines = std::max(1, kRepackThreads / row_words);
+    // the most rows of threads that fit, in as many trips, spread evenly over the trips: a trip
+    // goes past the slot's rows by fewer than kRepackUnroll rows a trip
+    const int most = std::max(1, kRepackThreads / row_words), trips = (v.rows - 1) / (kRepackUnroll * most) + 1;
+    const int lines = (v.rows - 1) / (kRepackUnroll * trips) + 1;
     const int block = (row_words * lines + 31) / 32 * 32;
     for (int l = 0; l < nlayers; l += 65535) {  // a grid's z limit
         const dim3 grid(v.nbx * v.nby, v.rows, std::min(nlayers - l, 65535));
