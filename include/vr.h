@@ -226,7 +226,7 @@ vr_status vr_render(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max, 
  * (termination is not differentiated); the forward is recomputed segment by
  * segment from per-segment checkpoints of T and swept back to front.  MIP:
  * the gradient reaches the first sample that attains the maximum.
- * Table partials are FP32 per block and summed in FP64.
+ * Table partials are FP32 per block (summed from its warps') and summed in FP64.
  * Errors as vr_render; VR_ERR_UNSUPPORTED (reported by the next call) if a
  * ray needs more than 320 checkpoint segments (about 10 000 samples).
  */

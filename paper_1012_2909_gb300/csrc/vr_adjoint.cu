@@ -12,9 +12,9 @@
 // the first pass keeps the transmittance at the start of every 32-sample chunk;
 // the reverse pass recomputes each chunk from its checkpoint, one sample per
 // lane, and gets (R_k, P_k) from a warp suffix scan carried from the chunks
-// behind.  Table gradients go ray by ray through fixed-point histograms into a copy
-// per block in shared memory, then to per-block partials that a final kernel sums in
-// FP64; voxel gradients are scattered through the trilinear weights with FP32 atomics.
+// behind.  Table gradients are collected ray by ray in a histogram per warp in shared
+// memory, added up per warp in device memory, and summed over the blocks in FP64 by a final
+// kernel; voxel gradients are scattered through the trilinear weights with FP32 atomics.
 // MIP: the image is TF(max v); the gradient reaches the first maximal sample.
 #include <algorithm>
 
@@ -29,9 +29,9 @@ namespace {
 constexpr int kAdjThreads = 128;
 constexpr int kAdjWarps = kAdjThreads / 32;
 constexpr int kAdjMaxChunks = 320;  // 32-sample transmittance checkpoints per ray
-constexpr int kAdjFlush = 8;        // chunks collected in the table histograms at a time
 constexpr int kAdjKeep = 6;         // chunks whose samples the forward pass keeps for the reverse pass
 constexpr int kDevTooManySegments = 2;
+constexpr int kAdjCrowd = 8;        // samples on one table interval that are reduced by the whole warp
 
 // Tables of up to kAdjTF entries and the default brick edge are compiled in (FAST): the
 // table's arrays are S entries apart, S = 0 standing for its length.
@@ -105,21 +105,78 @@ __device__ __forceinline__ void scatter_voxels(float* __restrict__ dvol, const V
     }
 }
 
-// g: the block's table gradient, channel-major (g[c * stride + i]), so that the lanes
-// of one atomic instruction fall on banks by table entry, not by entry mod 8.
-template <int S>
-__device__ __forceinline__ void add_tf(float* __restrict__ g, int n, const TFGrad& t, float4 gc) {
+// Adds w gc to one entry of a table gradient.
+__device__ __forceinline__ void add_entry(float4* g, float w, float4 gc) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(g), "f"(w * gc.x), "f"(w * gc.y),
+                 "f"(w * gc.z), "f"(w * gc.w)
+                 : "memory");
+}
+__device__ __forceinline__ void add_tf(float4* g, const TFGrad& t, float4 gc) {
+    add_entry(g + t.i, 1.f - t.w, gc);
+    add_entry(g + t.i + 1, t.w, gc);
+}
+
+// One sample a lane (act) into the warp's histogram: wk and ga are shared by the entries t.i
+// and t.i + 1 with weights 1 - t.w and t.w.  The lanes of one interval are added up first: by
+// a reduction over the warp where there are at least kAdjCrowd of them (regions of one value:
+// 256^3 with all below 3 sigma set to 0 and a fifth of the opacity, 23.5 ms a step, and 30.2 one
+// lane at a time; 6 the same, 4 costs 6 % on noise), else by the group's first lane, one mate
+// at a time (noise: 7.80 ms a step, and 7.93 with the lanes taking turns at the entries).  Each
+// interval then has one writer; lower entries are written before upper ones.
+__device__ __forceinline__ void collect_sample(float2* __restrict__ hist, const TFGrad& t, bool act, int lane,
+                                               float wk, float ga) {
+    constexpr unsigned int FULL = 0xffffffffu;
+    const unsigned int same = __match_any_sync(FULL, t.i);
     const float w1 = t.w, w0 = 1.f - t.w;
-    const int d = stride<S>(n);
-    float* a = g + t.i;
-    atomicAdd(a, w0 * gc.x);
-    atomicAdd(a + d, w0 * gc.y);
-    atomicAdd(a + 2 * d, w0 * gc.z);
-    atomicAdd(a + 3 * d, w0 * gc.w);
-    atomicAdd(a + 1, w1 * gc.x);
-    atomicAdd(a + d + 1, w1 * gc.y);
-    atomicAdd(a + 2 * d + 1, w1 * gc.z);
-    atomicAdd(a + 3 * d + 1, w1 * gc.w);
+    float c0 = w0 * wk, c1 = w1 * wk, a0 = w0 * ga, a1 = w1 * ga;
+    const bool crowd = act && __popc(same) >= kAdjCrowd;
+    for (unsigned int left = __ballot_sync(FULL, crowd); left;) {
+        const int first = __ffs(left) - 1;
+        const unsigned int group = __shfl_sync(FULL, same, first);
+        const bool in = (group >> lane) & 1u;
+        float4 v = in ? make_float4(c0, a0, c1, a1) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            v.x += __shfl_xor_sync(FULL, v.x, off);
+            v.y += __shfl_xor_sync(FULL, v.y, off);
+            v.z += __shfl_xor_sync(FULL, v.z, off);
+            v.w += __shfl_xor_sync(FULL, v.w, off);
+        }
+        if (lane == first) {
+            hist[t.i].x += v.x;
+            hist[t.i].y += v.y;
+            hist[t.i + 1].x += v.z;
+            hist[t.i + 1].y += v.w;
+        }
+        __syncwarp();
+        left &= ~group;
+    }
+    // the others: a group's first lane adds up its mates
+    const bool lead = act && !crowd && lane == __ffs(same) - 1;
+    unsigned int mates = lead ? same & (same - 1) : 0u;
+    const int rounds = __reduce_max_sync(FULL, __popc(mates));
+    for (int q = 0; q < rounds; ++q) {
+        const int src = mates ? __ffs(mates) - 1 : lane;
+        const float sw = __shfl_sync(FULL, w1, src), sk = __shfl_sync(FULL, wk, src), sg = __shfl_sync(FULL, ga, src);
+        if (mates) {
+            c0 = fmaf(1.f - sw, sk, c0);
+            c1 = fmaf(sw, sk, c1);
+            a0 = fmaf(1.f - sw, sg, a0);
+            a1 = fmaf(sw, sg, a1);
+        }
+        mates &= mates - 1;
+    }
+    // no two first lanes share an interval: lower entries, then upper ones
+    if (lead) {
+        hist[t.i].x += c0;
+        hist[t.i].y += a0;
+    }
+    __syncwarp();
+    if (lead) {
+        hist[t.i + 1].x += c1;
+        hist[t.i + 1].y += a1;
+    }
+    __syncwarp();
 }
 
 // One warp per ray, its lanes on 32 consecutive samples (a chunk).  A warp
@@ -139,27 +196,22 @@ __device__ __forceinline__ void add_tf(float* __restrict__ g, int n, const TFGra
 //
 // Table gradient.  A float atomicAdd in shared memory is a compare-and-swap loop,
 // repeated while lanes meet on an entry; eight a sample (4 channels x 2 entries) took
-// 30 % of the kernel.  Integer atomics are single instructions, and within one ray
-// everything is bounded, so a ray is collected in two 32-bit fixed-point histograms,
-// with four integer atomics a sample, and added to the block's FP32 copy once, over
-// the entries it touched:
-//   colour: dL/dc_k = dL/dC T_k a_k, one weight T_k a_k for all three channels; the
-//     weights of a ray add up to at most 1 and are kept in units of 2^-30;
-//   alpha: |dL/da_k| <= M = |g.w| + 2 cmax (|g.x| + |g.y| + |g.z|), cmax the table's
-//     largest colour; scaled by 2^-E, 2^E <= M < 2^(E+1), and kept in units of n / 2^29, n
-//     the samples collected together (at most 256 of a ray), so that no sum leaves 31
-//     bits.
-// A sample is rounded by 2^-22 M at most, less than the FP32 sums over the rays round.
-// This needs opacities in [0, 1] and a finite M; other tables, and rays whose dL/dI is
-// not finite, take the FP32 atomics.
+// 30 % of the kernel.  A ray is collected in a histogram of its warp instead, two values an
+// entry (dL/dc_k = dL/dC T_k a_k: one weight T_k a_k for all three channels, and dL/da_k),
+// without atomics: lanes whose samples fall between the same two entries are found by
+// __match_any_sync and added up in registers first (collect_sample).  Everything is FP32, so
+// a term keeps its 24 bits however small the transmittance before it is (histograms in fixed
+// point, with integer atomics, were 4 % faster over the step and lost the entries that are
+// reached only behind others; float atomics into the histograms were 14 % slower).  After a
+// ray, the entries touched go to the warp's gradient in device memory, a reduction of four
+// floats each: no copy of the table's gradient takes shared memory from the L1 cache (one a
+// warp there cost 25 % of the MIP gradient), and no sum runs over more rays than a warp's.
 //
 // Bound by L1 data wavefronts and the voxel atomics in L2 (both 78 % busy), with issue
 // slots at 63 %: two passes over a chunk took some 1100 warp instructions before the
 // anchors of a ray's chunks were made together, the default brick edge and table stride
 // compiled in, the voxel addresses taken from one base and aligned x-pairs reduced
-// together.  16 views of 512 x 512 on 256^3 FP32, forward and backward: 11.6 -> 7.2 ms (8.0
-// before these).  Five CTAs an SM and kAdjKeep = 6: 7.73 ms; six CTAs and 4: 7.79; five and
-// 4: 7.81 (one seed).
+// together.  16 views of 512 x 512 on 256^3 FP32, forward and backward (one seed): 11.85 -> 7.73 ms.  Six CTAs an SM and kAdjKeep = 4 instead of five and 6: the same.
 struct RaySetup {
     float o_hi[3], o_lo[3], e_hi[3], e_lo[3];
     int k0, k1;
@@ -227,21 +279,16 @@ __device__ __forceinline__ LaneSample lane_sample(const RaySetup& r, int c, int 
     return s;
 }
 
-constexpr float kColourUnits = 1073741824.f;  // 2^30
-constexpr float kAlphaUnits = 536870912.f;    // 2^29
-
 template <typename T, int MODE, bool FAST>
 __global__ void __launch_bounds__(kAdjThreads, 5)
 k_adjoint(const __grid_constant__ AdjParams P) {
     constexpr unsigned int FULL = 0xffffffffu;
-    // dynamic, by the size of the table: the table and the block's gradient of it, both
-    // channel-major, then a pair of histograms per warp
+    // dynamic, by the size of the table: the table, channel-major, and a histogram per warp
     extern __shared__ __align__(16) float s_dyn[];
     constexpr int S = FAST ? kAdjTF : 0, BR = FAST ? kFastBrick : 0;
     const int ntf = P.tf.n, sd = stride<S>(ntf);
     const Anchor slot0{0.f, 0.f, 0.f, 0};  // fetches from the slot's first voxel
     float* s_tf = s_dyn;
-    float* g_tf = s_dyn + 4 * sd;
     __shared__ RaySetup s_ray[kAdjWarps][32];
     __shared__ SampleAnchor s_anchor[kAdjWarps][32];
     __shared__ float2 s_keep[kAdjWarps][MODE == VR_COMPOSITE ? kAdjKeep * 32 : 1];
@@ -252,12 +299,12 @@ k_adjoint(const __grid_constant__ AdjParams P) {
         s_tf[2 * sd + i] = t.z;
         s_tf[3 * sd + i] = t.w;
     }
-    for (int i = threadIdx.x; i < (4 + (MODE == VR_COMPOSITE ? 2 * kAdjWarps : 0)) * sd; i += blockDim.x)
-        g_tf[i] = 0.f;
+    if (MODE == VR_COMPOSITE)
+        for (int i = threadIdx.x; i < 2 * kAdjWarps * sd; i += blockDim.x) s_dyn[4 * sd + i] = 0.f;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int* hist_c = reinterpret_cast<int*>(g_tf + 4 * sd) + warp * 2 * sd;
-    int* hist_a = hist_c + sd;
+    float2* hist = reinterpret_cast<float2*>(s_dyn + 4 * sd) + warp * sd;
+    float4* g_tf = P.tf_partials + (size_t)(blockIdx.x * kAdjWarps + warp) * ntf;  // this warp's gradient
     float2* keep = s_keep[warp];
     SampleAnchor* anchors = s_anchor[warp];
     const int tiles_per_cam = P.tiles_x * P.tiles_y;
@@ -331,7 +378,7 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                 if (kmax < 0) continue;
                 if (lane == 0) {
                     const TFGrad t = tf_eval<S>(s_tf, ntf, P.tf.vmin, P.tf.inv_range, m);
-                    add_tf<S>(g_tf, ntf, t, gI);
+                    add_tf(g_tf, t, gI);
                     if (P.dvol) {
                         SampleAnchor ls;
                         sample_anchor(r, kmax, P.vol, ls);
@@ -388,12 +435,7 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                 }
             }
             __syncwarp();
-            // fixed-point units of this ray's alpha gradients (see above)
-            const float bound = fabsf(gI.w) + 2.f * P.tf_cmax * (fabsf(gI.x) + fabsf(gI.y) + fabsf(gI.z));
-            const bool fixed = P.tf_unit && bound < 1e30f;
-            const float p2 = pow2_recip(bound);
-            const float to_units = kAlphaUnits / (float)min(32 * (nch - 1) + n_last, 32 * kAdjFlush);
-            const float from_units = 1.f / to_units / p2;
+            const bool collect = fabsf(gI.x) + fabsf(gI.y) + fabsf(gI.z) < INFINITY;  // NaN: false
             int e_lo = ntf, e_hi = 0;  // entries touched by this lane's samples
             // ---- reverse: chunks back to front, suffix "over" scan within a chunk
             float Rc = 0.f, Pc = 1.f;
@@ -402,6 +444,7 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                 const bool act = lane < n;
                 const float ckT = __shfl_sync(FULL, c < 32 ? ck0 : ck[(c >> 5) - 1], c & 31);
                 TFGrad t;
+                t.i = -1;
                 LaneSample ls;
                 if (c >= kAdjKeep || P.dvol) ls = lane_sample(r, c, lane, e32, P.vol, anchors, group);
                 float a = 0.f, s = 0.f, incl = 1.f;
@@ -451,70 +494,63 @@ k_adjoint(const __grid_constant__ AdjParams P) {
                 const float ha = __shfl_sync(FULL, A, 0), hb = __shfl_sync(FULL, Bq, 0);
                 Rc = fmaf(hb, Rc, ha);
                 Pc *= hb;
-                if (act) {
-                    const float wk = Tin * a;
-                    const float ga = gI.w * Tin * Pt + Tin * (s - R);
-                    if (fixed) {
-                        const float w1 = t.w, w0 = 1.f - t.w;
-                        const float hw = wk * kColourUnits, hg = (ga * p2) * to_units;
-                        atomicAdd(hist_c + t.i, __float2int_rn(w0 * hw));
-                        atomicAdd(hist_c + t.i + 1, __float2int_rn(w1 * hw));
-                        atomicAdd(hist_a + t.i, __float2int_rn(w0 * hg));
-                        atomicAdd(hist_a + t.i + 1, __float2int_rn(w1 * hg));
+                const float wk = Tin * a;
+                const float ga = gI.w * Tin * Pt + Tin * (s - R);
+                if (collect) {
+                    collect_sample(hist, t, act, lane, wk, ga);
+                    if (act) {
                         e_lo = min(e_lo, t.i);
                         e_hi = max(e_hi, t.i + 1);
-                    } else {
-                        add_tf<S>(g_tf, ntf, t, make_float4(gI.x * wk, gI.y * wk, gI.z * wk, ga));
                     }
+                } else if (act) {
+                    add_tf(g_tf, t, make_float4(gI.x * wk, gI.y * wk, gI.z * wk, ga));
+                }
+                if (act) {
                     if (P.dvol) {
                         const float dv = wk * (gI.x * t.slope.x + gI.y * t.slope.y + gI.z * t.slope.z) + ga * t.slope.w;
                         scatter_voxels(P.dvol, P.vol, ls.bx, ls.by, ls.bz, ls.gx, ls.gy, ls.gz, dv);
                     }
                 }
-                if (fixed && c % kAdjFlush == 0) {  // the histograms, over the entries touched, to the block's copy
-                    __syncwarp();
-                    e_lo = __reduce_min_sync(FULL, e_lo);
-                    e_hi = __reduce_max_sync(FULL, e_hi);
-                    for (int e = e_lo + lane; e <= e_hi; e += 32) {
-                        const int hc = hist_c[e], hg = hist_a[e];
-                        if (hc | hg) {
-                            hist_c[e] = 0;
-                            hist_a[e] = 0;
-                            const float h = (float)hc * (1.f / kColourUnits);
-                            atomicAdd(g_tf + e, gI.x * h);
-                            atomicAdd(g_tf + sd + e, gI.y * h);
-                            atomicAdd(g_tf + 2 * sd + e, gI.z * h);
-                            atomicAdd(g_tf + 3 * sd + e, (float)hg * from_units);
-                        }
+            }
+            if (collect) {  // the histogram, over the entries touched, to the warp's partial
+                e_lo = __reduce_min_sync(FULL, e_lo);
+                e_hi = __reduce_max_sync(FULL, e_hi);
+                for (int e = e_lo + lane; e <= e_hi; e += 32) {
+                    const float2 h = hist[e];
+                    if (h.x != 0.f || h.y != 0.f) {
+                        hist[e] = make_float2(0.f, 0.f);
+                        add_entry(g_tf + e, 1.f, make_float4(gI.x * h.x, gI.y * h.x, gI.z * h.x, h.y));
                     }
-                    e_lo = ntf;
-                    e_hi = 0;
-                    __syncwarp();
                 }
             }
             __syncwarp();
         }
         __syncwarp();  // the tile's ray set-ups are read before the next tile overwrites them
     }
-    __syncthreads();
-    // block partial, entry-major (ntf x 4)
-    float* out = P.tf_partials + (size_t)blockIdx.x * ntf * 4;
-    for (int i = threadIdx.x; i < ntf * 4; i += blockDim.x) out[i] = g_tf[(i & 3) * sd + (i >> 2)];
 }
 
-// Final reduction of the per-block table partials, in FP64 (the only FP64
-// arithmetic on the gradient path).
-// A block per 32 values, its warps on interleaved blocks' partials (a thread a value,
-// serial over the partials, took 121 us for 760 x 1024: four blocks in all).
-constexpr int kReduceWarps = 16;
+// Final reduction of the table gradients of the warps, nblocks x kAdjWarps x nval: a block's
+// in FP32, over the blocks in FP64 (the only FP64 arithmetic on the gradient path; all rows in
+// FP64 took 58 us for 3040 x 1024).
+// A block per 32 values, its warps on interleaved blocks' rows (a thread a value, serial over
+// the rows, took 121 us for 760 x 1024: four blocks in all).
+constexpr int kReduceWarps = 32;
 __global__ void __launch_bounds__(kReduceWarps * 32)
 k_tfgrad_reduce(const float* __restrict__ partials, int nblocks, int nval, float* __restrict__ out) {
     __shared__ double s_acc[kReduceWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
     double acc = 0.0;
-    if (i < nval)
-        for (int b = warp; b < nblocks; b += kReduceWarps) acc += (double)partials[(size_t)b * nval + i];
+    if (i < nval) {
+#pragma unroll 4
+        for (int b = warp; b < nblocks; b += kReduceWarps) {
+            const float* p = partials + (size_t)b * kAdjWarps * nval + i;
+            float v = p[0];
+#pragma unroll
+            for (int w = 1; w < kAdjWarps; ++w) v += p[(size_t)w * nval];
+            acc += (double)v;
+        }
+    }
     s_acc[warp][lane] = acc;
     __syncthreads();
     if (warp == 0 && i < nval) {
@@ -532,10 +568,10 @@ void* adj_t(int mode, bool fast) {
                 : reinterpret_cast<void*>(&k_adjoint<T, VR_COMPOSITE, false>);
 }
 
-// The kernel for p and its dynamic shared memory: table, its gradient, two histograms a warp.
+// The kernel for p and its dynamic shared memory: the table, and a histogram a warp.
 void* adj_pick(const AdjParams& p, vr_dtype dt, size_t& smem) {
     const bool fast = p.vol.B == kFastBrick && p.tf.n <= kAdjTF;
-    smem = (size_t)(fast ? kAdjTF : p.tf.n) * sizeof(float) * (8 + (p.mode == VR_COMPOSITE ? 2 * kAdjWarps : 0));
+    smem = (size_t)(fast ? kAdjTF : p.tf.n) * sizeof(float) * (4 + (p.mode == VR_COMPOSITE ? 2 * kAdjWarps : 0));
     void* f = dt == VR_F32   ? adj_t<float>(p.mode, fast)
               : dt == VR_F16 ? adj_t<__half>(p.mode, fast)
                              : adj_t<__nv_bfloat16>(p.mode, fast);
@@ -543,6 +579,8 @@ void* adj_pick(const AdjParams& p, vr_dtype dt, size_t& smem) {
 }
 
 }  // namespace
+
+int adjoint_warps() { return kAdjWarps; }
 
 int adjoint_blocks_per_sm(const AdjParams& p, vr_dtype dt) {
     size_t smem;
@@ -560,8 +598,10 @@ cudaError_t launch_adjoint(const AdjParams& p, vr_dtype dt, int grid, cudaStream
     return cudaLaunchKernel(f, dim3(grid), dim3(kAdjThreads), args, smem, s);
 }
 
-cudaError_t launch_tfgrad_reduce(const float* partials, int nblocks, int nval, float* out, cudaStream_t s) {
-    k_tfgrad_reduce<<<(nval + 31) / 32, kReduceWarps * 32, 0, s>>>(partials, nblocks, nval, out);
+cudaError_t launch_tfgrad_reduce(const float4* partials, int nblocks, int ntf, float* out, cudaStream_t s) {
+    const int nval = 4 * ntf;
+    k_tfgrad_reduce<<<(nval + 31) / 32, kReduceWarps * 32, 0, s>>>(reinterpret_cast<const float*>(partials), nblocks,
+                                                                   nval, out);
     return cudaGetLastError();
 }
 

@@ -101,7 +101,7 @@ struct vr_ctx {
     long long partial_cap = 0;
     float4* state = nullptr;
     long long state_cap = 0;
-    float* tf_partials = nullptr;  // adjoint: per-block table-gradient partials
+    float4* tf_partials = nullptr;  // adjoint: table gradients of the warps
     size_t tf_partials_n = 0;
     int* status_host = nullptr;    // mapped, page-locked device status word
     int* status_dev = nullptr;
@@ -1709,25 +1709,25 @@ vr_status vr_render_backward(vr_ctx* ctx, vr_mode mode, const float* dL_dimg, fl
     P.tiles_y = (P.height + kTileH - 1) / kTileH;
     split(ctx->opt.step, P.step_hi, P.step_lo);
     P.ert = (float)ctx->opt.ert;
-    P.tf_unit = 1;
-    for (const float4& t : ctx->tf) {
-        if (!(t.w >= 0.f && t.w <= 1.f)) P.tf_unit = 0;
-        P.tf_cmax = std::max(P.tf_cmax, std::max(std::fabs(t.x), std::max(std::fabs(t.y), std::fabs(t.z))));
-    }
     P.dvol = dL_dvol;
     P.status = ctx->status_dev;
-    const int grid = ctx->num_sms * adjoint_blocks_per_sm(P, ctx->dtype);
-    const size_t need = (size_t)nbatch * grid * ntf * 4;
+    // persistent blocks, no more than there are tiles for their warps; a partial table a warp
+    const int warps = adjoint_warps();
+    const long long tiles = (long long)P.tiles_x * P.tiles_y * std::min(ncams, kMaxLaunchCams);
+    const int grid = (int)std::min<long long>(ctx->num_sms * adjoint_blocks_per_sm(P, ctx->dtype),
+                                              (tiles + warps - 1) / warps);
+    const size_t need = (size_t)nbatch * grid * warps * ntf;
     if (need > ctx->tf_partials_n) {
         if (ctx->tf_partials) cudaFree(ctx->tf_partials);
         ctx->tf_partials = nullptr;
         ctx->tf_partials_n = 0;
-        VR_CK(cudaMalloc(&ctx->tf_partials, need * sizeof(float)), "vr_render_backward: partials");
+        VR_CK(cudaMalloc(&ctx->tf_partials, need * sizeof(float4)), "vr_render_backward: partials");
         ctx->tf_partials_n = need;
     }
     if (dL_dvol)
         VR_CK(cudaMemsetAsync(dL_dvol, 0, sizeof(float) * (size_t)ctx->nx * ctx->ny * ctx->nz, s),
               "vr_render_backward: clear dL_dvol");
+    VR_CK(cudaMemsetAsync(ctx->tf_partials, 0, need * sizeof(float4), s), "vr_render_backward: clear partials");
     VR_CK(cudaMemsetAsync(ctx->work, 0, sizeof(int) * nbatch, s), "vr_render_backward: scheduler reset");
     const long long img = (long long)P.width * P.height;
     for (int b = 0; b < nbatch; ++b) {
@@ -1735,11 +1735,11 @@ vr_status vr_render_backward(vr_ctx* ctx, vr_mode mode, const float* dL_dimg, fl
         P.ncams = std::min(kMaxLaunchCams, ncams - c0);
         for (int i = 0; i < P.ncams; ++i) P.cams[i] = ray_cam(ctx->cams[(size_t)(c0 + i)]);
         P.dimg = reinterpret_cast<const float4*>(dL_dimg) + (long long)c0 * img;
-        P.tf_partials = ctx->tf_partials + (size_t)b * grid * ntf * 4;
+        P.tf_partials = ctx->tf_partials + (size_t)b * grid * warps * ntf;
         P.work = ctx->work + b;
         VR_CK(launch_adjoint(P, ctx->dtype, grid, s), "vr_render_backward: adjoint launch");
     }
-    VR_CK(launch_tfgrad_reduce(ctx->tf_partials, nbatch * grid, ntf * 4, dL_dtf, s),
+    VR_CK(launch_tfgrad_reduce(ctx->tf_partials, nbatch * grid, ntf, dL_dtf, s),
           "vr_render_backward: table reduction");
     return VR_OK;
 }

@@ -124,11 +124,10 @@ struct AdjParams {
     int tiles_x, tiles_y;
     float step_hi, step_lo;  // the sample spacing as a float-float pair
     float ert;
-    int tf_unit;          // every opacity of the table is in [0, 1]
-    float tf_cmax;        // its largest colour magnitude
+    int pad2;
     const float4* dimg;   // dL/dI of camera 0 of this launch
     float* dvol;          // dL/dvoxel, linear x-fastest (may be null)
-    float* tf_partials;   // per-block table partials of this launch (grid x ntf x 4)
+    float4* tf_partials;  // zeroed table gradients of this launch's warps (grid x warps x ntf)
     int* work;            // zeroed work counter of this launch
     int* status;          // device status word
 };
@@ -271,9 +270,10 @@ long long pyramid_levels(int w, int h, int tlog2, std::vector<int>& ws, std::vec
 cudaError_t launch_pyramid(const float4* in, int w, int h, int tlog2, float4* out, cudaStream_t s);
 // Bounded-wait self-test (vr_selftest.cu): one waiter that gives up after `polls`.
 cudaError_t launch_wait_probe(int* status, unsigned long long limit_ns, cudaStream_t s);
+int adjoint_warps();  // warps of a block
 int adjoint_blocks_per_sm(const AdjParams& p, vr_dtype dt);
 cudaError_t launch_adjoint(const AdjParams& p, vr_dtype dt, int grid, cudaStream_t s);
-cudaError_t launch_tfgrad_reduce(const float* partials, int nblocks, int nval, float* out, cudaStream_t s);
+cudaError_t launch_tfgrad_reduce(const float4* partials, int nblocks, int ntf, float* out, cudaStream_t s);
 // Brick-path MIP pieces used by the allocation-free entry point (vr_api.cu).
 vr_status brick_mip_precheck(vr_ctx* ctx, float* out_rgba, float* out_max, int* device,
                              long long* pixels);
