@@ -239,9 +239,12 @@ vr_status vr_render_backward(vr_ctx* ctx, vr_mode mode, const float* dL_dimg, fl
  *   block:           threads per CTA of the image-order path (64, 128, 256);
  *   group:           lanes per ray segment in the brick path (4, 8, 16), i.e.
  *                    32 / group rays per warp.
- * Defaults 8 x 4, 256, 8; until a tuning is set, the brick path takes 4 lanes
- * instead where the rays are dense (with FP32 cells also where less so).  Results do not
- * depend on the tuning (up to rounding). */
+ * Defaults 8 x 4, 256, 8.  The brick path takes 4 lanes instead of 8 where the rays
+ * are dense (with FP32 cells also where less so) until lanes are chosen: by
+ * vr_autotune over the brick path, or by vr_set_tuning with a group other than the
+ * one that vr_get_tuning reports (setting back what was read, or with another
+ * tile or block, chooses none).  Results do not depend on the tuning (up to
+ * rounding). */
 typedef struct {
     int32_t tile_w, tile_h;
     int32_t block;

@@ -562,6 +562,8 @@ def autotune(renderer: Renderer, mode: str, reps: int = 5, cache: str | None = N
         with open(cache) as f:
             table = json.load(f)
     if key in table:
+        if mode == "mip":  # its lanes were measured: held also where they are the ones reported
+            vr_set_tuning(renderer.ctx, dict(table[key], group=4 if table[key]["group"] != 4 else 8))
         vr_set_tuning(renderer.ctx, table[key])
         return dict(table[key], cached=True)
     scratch = torch.empty((n, h, w, 4), dtype=torch.float32, device=renderer.torch_device)

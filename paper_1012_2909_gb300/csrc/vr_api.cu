@@ -1609,8 +1609,9 @@ vr_status vr_set_tuning(vr_ctx* ctx, const vr_tuning* t) {
     if (!tuning_ok(*t))
         return fail(ctx, VR_ERR_INVALID_ARG,
                     "vr_set_tuning: need tile_w * tile_h == 32, block in {64,128,256}, group in {4,8,16}");
+    // the lanes reported, set back with or without another tile or block, are no choice of lanes
+    ctx->group_set |= t->group != ctx->tune.group;
     ctx->tune = *t;
-    ctx->group_set = true;
     return VR_OK;
 }
 
