@@ -17,6 +17,7 @@
 #include <cudaTypedefs.h>
 
 #include "vr_internal.cuh"
+#include "vr_pass.cuh"
 #include "vr_tma.cuh"
 
 using namespace vr;
@@ -843,38 +844,13 @@ FinalizeParams finalize_params(const vr_ctx* ctx) {
     return p;
 }
 
-// Area of a pixel, in square voxels, at the cube's centre.
-double pixel_area(const vr_ctx* ctx, const CamDev& cd) {
+// Shape of a staged-cell pass over n cameras: the rule's, with the lanes that the caller or
+// the autotuner chose.
+PassShape pass_shape(const vr_ctx* ctx, const CamDev* cams, int n) {
     const double c[3] = {0.5 * (double)ctx->nx, 0.5 * (double)ctx->ny, 0.5 * (double)ctx->nz};
-    auto len2 = [](const double* v) { return v[0] * v[0] + v[1] * v[1] + v[2] * v[2]; };
-    double scale = 1.0;  // of the window at the cube's centre
-    if (cd.type == 1) {
-        scale = 0.0;
-        for (int a = 0; a < 3; ++a) scale += (c[a] - cd.eye[a]) * cd.fwd[a];
-        scale = std::fabs(scale) / len2(cd.fwd);
-    }
-    return std::fabs(cd.du * cd.dv) * std::sqrt(len2(cd.right) * len2(cd.up)) * scale * scale;
-}
-
-// Lanes per ray segment of a staged-cell pass over views like `cd`: the tuning's where the
-// caller or the autotuner set one, else by the length of the segments and the spacing of
-// the rays at the cube's centre.  Fewer lanes waste less on a segment's last step, and pay
-// where neighbouring groups march segments of one length: in the short segments of FP32
-// cells (16 voxels thick: 1721 x 1721 x 1025 at 1.0 voxels a pixel 18.9 ms with 4 lanes and
-// 19.7 with 8; equal within 1 % up to 3 voxels a pixel; 1269 x 339 x 736 at 7.8 voxels a
-// pixel 0.313 and 0.301; not measured between), and with 16-bit cells where the rays are
-// at most a voxel apart (2048 x 2048 x 1024 on 25 panels: 0.66 voxels 49.4 and
-// 53.3 ms, 0.99 25.6 and 26.0; 1.31 16.6 and 16.3; 1024 x 1024 x 2048 at 2.7 voxels 2.57 and 2.27).
-int pass_group(const vr_ctx* ctx, const CamDev& cd) {
-    if (ctx->group_set) return ctx->tune.group;
-    return pixel_area(ctx, cd) <= (ctx->dtype == VR_F32 ? 9.0 : 1.0) ? 4 : 8;
-}
-
-// Most row bands of a staged cell's pixels (BrickParams::max_bands): a 32^3 cell covers
-// some 1500 square voxels, and a band should keep 512 pixels.
-int pass_bands(const vr_ctx* ctx, const CamDev& cd) {
-    const double px = 1500.0 / std::max(pixel_area(ctx, cd), 1e-3);
-    return (int)std::min(64.0, std::max(1.0, px / 512.0));
+    PassShape p = pass_rule(c, cams, n, ctx->dtype == VR_F32);
+    if (ctx->group_set) p.group = ctx->tune.group;
+    return p;
 }
 
 // MIP through the brick pass, up to kMaxLaunchCams cameras per pass over the
@@ -917,7 +893,8 @@ vr_status render_brick_mip(vr_ctx* ctx, float* out_rgba, float* out_max, cudaStr
             pp.cams[i] = bp.cams[i];
         }
         bp.out_enc = enc;
-        bp.max_bands = pass_bands(ctx, ctx->cams[(size_t)c0]);
+        const PassShape shape = pass_shape(ctx, &ctx->cams[(size_t)c0], nb);
+        bp.max_bands = shape.bands;
         bp.work = ctx->work + kMaxLaunchCams + (c0 / per) % 4096;
         pp.ncams = nb;
         pp.enc = enc;
@@ -925,9 +902,7 @@ vr_status render_brick_mip(vr_ctx* ctx, float* out_rgba, float* out_max, cudaStr
         pp.zero[1] = static_cast<int*>(ctx->cells);
         VR_CK(launch_pixel_setup(pp, s), "vr_render: pixel set-up");
         if (c0 == 0 && ctx->ev_start) VR_CK(cudaEventRecord(ctx->ev_start, s), "vr_render: profiling event");
-        VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, grid, ctx->cells, s,
-                               pass_group(ctx, ctx->cams[(size_t)c0])),
-              "vr_render: brick pass");
+        VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, grid, ctx->cells, s, shape.group), "vr_render: brick pass");
         if (c0 + nb >= ncams && ctx->ev_stop) VR_CK(cudaEventRecord(ctx->ev_stop, s), "vr_render: profiling event");
         fp.npix = (long long)nb * img;
         fp.enc = enc;
@@ -994,7 +969,8 @@ vr_status staged_partials(vr_ctx* ctx, const CamDev& cd, const SortParams& sp, i
     bp.status = ctx->status_dev;
     bp.brick_list = brick_list;
     bp.nlist = nlist;
-    bp.max_bands = pass_bands(ctx, cd);
+    const PassShape shape = pass_shape(ctx, &cd, 1);
+    bp.max_bands = shape.bands;
     bp.foot = sp.foot;
     bp.partial = sp.partial;
     bp.key_persp = cd.type == 1;
@@ -1004,7 +980,7 @@ vr_status staged_partials(vr_ctx* ctx, const CamDev& cd, const SortParams& sp, i
     }
     VR_CK(launch_cell_partials(&ctx->tmap_part, bp, sp.tf, ctx->dtype, mode, npartial,
                                cell_partial_passes(ctx->dtype, ctx->B), 2 * ctx->num_sms, ctx->cells, s,
-                               pass_group(ctx, cd)),
+                               shape.group),
           "sort-last partial images");
     *done = true;
     return VR_OK;
@@ -1317,7 +1293,7 @@ vr_status render_ooc(vr_ctx* ctx, vr_mode mode, float* out_rgba, float* out_max,
                 VR_CK(cudaMemsetAsync(bp.work, 0, sizeof(int), s), "out of core: scheduler reset");
                 VR_CK(cudaMemsetAsync(ctx->cells, 0, sizeof(int), s), "out of core: cell count reset");
                 VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s,
-                                       pass_group(ctx, cd)),
+                                       pass_shape(ctx, &cd, 1).group),
                       "out of core: brick pass");
             }
             VR_CK(launch_mip_finalize(fp, s), "out of core: finalise");
@@ -1452,11 +1428,10 @@ vr_status brick_mip_with_scratch(vr_ctx* ctx, float* out_rgba, float* out_max, c
         fp.out_rgba = reinterpret_cast<float4*>(out_rgba) + (long long)i * img;
         fp.out_max = out_max ? out_max + (long long)i * img : nullptr;
         bp.out_enc = enc;
-        bp.max_bands = pass_bands(ctx, ctx->cams[(size_t)i]);
+        const PassShape shape = pass_shape(ctx, &ctx->cams[(size_t)i], 1);
+        bp.max_bands = shape.bands;
         VR_CK(launch_pixel_setup(pp, s), "pixel set-up");
-        VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s,
-                               pass_group(ctx, ctx->cams[(size_t)i])),
-              "brick pass");
+        VR_CK(launch_brick_mip(&ctx->tmap, bp, ctx->dtype, 2 * ctx->num_sms, ctx->cells, s, shape.group), "brick pass");
         VR_CK(launch_mip_finalize(fp, s), "finalise");
     }
     return VR_OK;
