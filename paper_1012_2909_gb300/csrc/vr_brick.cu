@@ -741,9 +741,9 @@ k_brick_mip(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ Br
 // of the ray's samples that the brick owns (the maximum of their values for
 // MIP).  The brick's cells split those samples by the same face-crossing rule,
 // so the partial is the front-to-back fold of the pixel's cell segments.  Each
-// visibility pass stages the cells of one local key (k_cell_list), marches each
-// segment with G lanes on consecutive samples, and folds the segment into the brick's slot: C += T C_seg, T *= T_seg
-// (or the maximum).  Slots start as the empty image (0, 0, 0, 1), or -inf.
+// visibility pass stages the cells of one local key (k_keyed_cells), marches each
+// segment with G lanes on consecutive samples, and folds the segment into the brick's
+// slot: C += T C_seg, T *= T_seg (or the maximum).  Slots start as the empty image (0, 0, 0, 1), or -inf.
 
 // Staged box without spare rows (the partial pass also holds the table).
 template <typename T> struct PartGeom {

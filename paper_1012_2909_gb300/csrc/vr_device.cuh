@@ -253,32 +253,6 @@ template <> __device__ __forceinline__ float2 ld_pair<__nv_bfloat16>(const __nv_
     return __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p) + w));
 }
 
-// fetch_trilinear with the four x-neighbour pairs read by one aligned load each:
-// element i of the slot starts word i / 2 of the store when i is even and word
-// i / 2 of the copy shifted by one element (slot1) when i is odd.  The row pitch
-// is even, so the parity of i is that of x.  Same operations on the same values
-// as fetch_trilinear, so the same result bit for bit.
-template <typename T>
-__device__ __forceinline__ float fetch_trilinear_pair(const T* __restrict__ slot, const T* __restrict__ slot1,
-                                                      const VolDev& v, float gx, float gy, float gz) {
-    const float B = (float)v.B;
-    gx = fminf(fmaxf(gx, 0.f), B + 0.999f);
-    gy = fminf(fmaxf(gy, 0.f), B + 0.999f);
-    gz = fminf(fmaxf(gz, 0.f), B + 0.999f);
-    const float fx0 = floorf(gx), fy0 = floorf(gy), fz0 = floorf(gz);
-    const float fx = gx - fx0, fy = gy - fy0, fz = gz - fz0;
-    const int ix = (int)fx0, iy = (int)fy0, iz = (int)fz0;
-    const int w = ((iz * v.rows + iy) * v.pitch + ix) >> 1;
-    const int hp = v.pitch >> 1, hs = (v.rows * v.pitch) >> 1;  // a row and a slab in words
-    const T* p = (ix & 1) ? slot1 : slot;
-    const float2 c00 = ld_pair<T>(p, w), c10 = ld_pair<T>(p, w + hp);
-    const float2 c01 = ld_pair<T>(p, w + hs), c11 = ld_pair<T>(p, w + hs + hp);
-    const float a0 = fmaf(fx, c00.y - c00.x, c00.x), a1 = fmaf(fx, c10.y - c10.x, c10.x);
-    const float a2 = fmaf(fx, c01.y - c01.x, c01.x), a3 = fmaf(fx, c11.y - c11.x, c11.x);
-    const float b0 = fmaf(fy, a1 - a0, a0), b1 = fmaf(fy, a3 - a2, a2);
-    return fmaf(fz, b1 - b0, b0);
-}
-
 // Sub-anchor of a ray inside a segment: the sample k's slot coordinate g = G + q0
 // split into an integer corner G (as the element offset `base` of voxel G in the
 // slot) and a remainder q0 in [0, 1] rounded once from float-float.  The samples
@@ -365,7 +339,10 @@ __device__ __forceinline__ float fetch_near(const T* __restrict__ slot, const Vo
     return fmaf(fz, b1 - b0, b0);
 }
 
-// fetch_trilinear_pair at slot coordinate G + q for the anchor's G (see fetch_near).
+// fetch_near with the four x-neighbour pairs read by one aligned load each: element i of the
+// slot starts word i / 2 of the store when i is even and word i / 2 of the copy shifted by one
+// element (slot1) when i is odd.  The row pitch is even, so the parity of i is that of x.  Same
+// operations on the same values as fetch_near, so the same result bit for bit.
 template <typename T, int BR>
 __device__ __forceinline__ float fetch_near_pair(const T* __restrict__ slot, const T* __restrict__ slot1,
                                                  const VolDev& v, const Anchor& A, float qx, float qy, float qz) {
