@@ -17,7 +17,7 @@
 #include <cudaTypedefs.h>
 
 #include "vr_internal.cuh"
-#include "vr_pass.cuh"
+#include "vr_pass.h"
 #include "vr_tma.cuh"
 
 using namespace vr;

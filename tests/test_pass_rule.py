@@ -11,7 +11,7 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 SOURCE = """
-#include "vr_pass.cuh"
+#include "vr_pass.h"
 extern "C" void shape(const double* spacing, int n, int f32, int* out) {
     const double c[3] = {32, 32, 32};
     std::vector<vr::CamDev> cams((size_t)n);
