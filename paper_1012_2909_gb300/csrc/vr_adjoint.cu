@@ -202,13 +202,13 @@ __device__ __forceinline__ void collect_sample(float2* __restrict__ hist, const 
 // __match_any_sync and added up in registers first (collect_sample).  Everything is FP32, so
 // a term keeps its 24 bits however small the transmittance before it is (histograms in fixed
 // point, with integer atomics, were 4 % faster over the step and lost the entries that are
-// reached only behind others; float atomics into the histograms were 14 % slower).  After a
+// reached only behind others; float atomics into the histograms were 13 % slower).  After a
 // ray, the entries touched go to the warp's gradient in device memory, a reduction of four
 // floats each: no copy of the table's gradient takes shared memory from the L1 cache (one a
-// warp there cost 25 % of the MIP gradient), and no sum runs over more rays than a warp's.
+// warp there made the MIP gradient a third slower), and no sum runs over more rays than a warp's.
 //
-// Bound by L1 data wavefronts and the voxel atomics in L2 (both 78 % busy), with issue
-// slots at 63 %: two passes over a chunk took some 1100 warp instructions before the
+// Bound by L1 data wavefronts (86 % busy) and the voxel reductions in L2 (70 %), with issue
+// slots at 55 % (8 views): two passes over a chunk took some 1100 warp instructions before the
 // anchors of a ray's chunks were made together, the default brick edge and table stride
 // compiled in, the voxel addresses taken from one base and aligned x-pairs reduced
 // together.  16 views of 512 x 512 on 256^3 FP32, forward and backward (one seed): 11.85 -> 7.73 ms.  Six CTAs an SM and kAdjKeep = 4 instead of five and 6: the same.

@@ -33,7 +33,9 @@ constexpr int kMarchUnrollPaired = 6;
 // view, lanes that wait for their neighbours included.  With constant slot offsets, no
 // clamps, rises and a termination without branches it takes 111: 128^3 FP32 at 512 x 512
 // 89.6 -> 77.1 us, 1721 x 1721 x 1025 FP32 at 3000 x 3000 3.27 -> 2.83 ms, survey FP16
-// 0.440 -> 0.412 ms, the same images bit for bit.
+// 0.440 -> 0.412 ms, the same images bit for bit.  (The times of a composite move with the seed
+// of the cube's noise by some 15 %: the two figures of a comparison share a seed and a run, those
+// of different comparisons here need not.)
 constexpr int kMarchTF = 256;
 
 // Asks L2 for what a sample some way ahead reads (both slabs; the offset is kept in the

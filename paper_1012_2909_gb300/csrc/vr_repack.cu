@@ -75,7 +75,7 @@ template <> struct Range<float> {
 // place of a device-to-device copy at a 2-byte offset afterwards.  Neighbouring bricks
 // read the ghost planes and row ends again, so the loads go through L2 as usual: with
 // streaming loads the survey cube (1024 x 1024 x 2048, 16-bit with the copy: 18.0 GB)
-// read 10.9 GB instead of 9.0.  That cube in 3.15 ms, 5.85 TB/s; before, 16 launches
+// read 10.9 GB instead of 8.6.  That cube in 3.09 ms, 5.82 TB/s; before, 16 launches
 // with an element a thread took 5.2 ms and the offset copy came on top (load and first
 // frame 15.4 -> 10.6 ms).  kRepackUnroll = 2, 8: the same, +10 %.
 constexpr int kRepackUnroll = 4;
